@@ -353,13 +353,14 @@ int dqmc_set_gemm_mode(dqmc_ctx* ctx, int mode);
 
 /* QR factorisation of the UDV stack steps (Sec. 2, the stabilisation of
  * Eq. (3)):
- *   DQMC_QR_BLOCKED (default): the columns of each step's product are sorted
- *     by decreasing norm once (pre-pivoting), then factorised without further
- *     pivoting by blocked Householder QR: FP64 panels of 32 columns, the
- *     trailing updates and the accumulation of Q on the tensor-core FP64
- *     products.  Used where those products are (DQMC_GEMM_TENSOR, N >= 64).
+ *   DQMC_QR_BLOCKED (default): for N > 144 the columns not yet factorised are
+ *     sorted by decreasing norm at the start of every panel and pivoted within
+ *     it: FP64 panels of 32 columns, the trailing updates and the accumulation
+ *     of Q on the tensor-core FP64 products.  Used where those products are
+ *     (DQMC_GEMM_TENSOR).
  *   DQMC_QR_PIVOTED: Householder QR with column pivoting on the FP64 pipe
- *     (always used for N < 64 and in DQMC_GEMM_FP64 mode).
+ *     (always used for N <= 144, where the matrix stays in shared memory, and
+ *     in DQMC_GEMM_FP64 mode).
  * Both give X = U D T with |diag| T = 1; G agrees between them to the
  * conditioning of the problem.  Drops captured sweep graphs.  Errors:
  * DQMC_ERR_ARG. */

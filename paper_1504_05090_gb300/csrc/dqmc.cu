@@ -329,11 +329,16 @@ cudaError_t gemm(dqmc_ctx* ctx, Group& g, const GemmArgs& m, int batch) {
 }
 
 // QR of the stack step X = B..B (U D) (rows of g.X = columns of X) into the
-// stack entry (Q^T at Qt, D at Dv) and g.Rtil: the blocked, pre-pivoted QR
-// with tensor-core updates where the tensor-core products are in use, the
-// column-pivoted cluster QR on the FP64 pipe otherwise.
+// stack entry (Q^T at Qt, D at Dv) and g.Rtil: column-pivoted with the matrix
+// in shared memory up to N = 144 (qr_smem_ctas), else the blocked QR with
+// tensor-core updates where the tensor-core products are in use, else the
+// column-pivoted cluster QR on global memory.
 cudaError_t stack_qr(dqmc_ctx* ctx, Group& g, double* Qt, double* Dv) {
   const long long sD = static_cast<long long>(g.nc + 1) * g.N;
+  const int cs = qr_smem_ctas(g.N, ctx->total, ctx->nsm);
+  if (cs > 0)
+    return launch_qr_smem(cs, g.X, g.nn(), Qt, g.sstride(), Dv, sD, g.Rtil, g.nn(), g.N, g.C,
+                          ctx->d_status, g.st);
   if (ctx->gemm_mode == DQMC_GEMM_TENSOR && ctx->qr_mode == DQMC_QR_BLOCKED && g.oz) {
     ctx->launches += qr_blocked_launches(g.N, g.C, g.oz_batch) - 1;
     return launch_qr_blocked(g.X, g.nn(), Qt, g.sstride(), Dv, sD, g.Rtil, g.nn(), g.qrb, g.N, g.C,
@@ -811,6 +816,7 @@ int dqmc_init_at(const dqmc_group* groups, int n_groups, uint64_t seed, int64_t 
   ctx->seed = seed;
   ctx->chain_offset = chain_offset;
   ctx->nsm = prop.multiProcessorCount;
+  for (int i = 0; i < n_groups; ++i) ctx->total += groups[i].n_chains;
   ctx->g.resize(n_groups);
   int rc = dev_alloc(ctx, &ctx->d_sweep, sizeof(uint32_t));
   if (rc == DQMC_OK) rc = dev_alloc(ctx, &ctx->d_status, sizeof(int));
@@ -840,7 +846,6 @@ int dqmc_init_at(const dqmc_group* groups, int n_groups, uint64_t seed, int64_t 
     if (rc == DQMC_OK) rc = rebuild(ctx, g);
     if (rc == DQMC_OK) rc = load_working(ctx, g);
   }
-  ctx->total = chain0;
   if (rc == DQMC_OK) {
     if (cudaStreamCreateWithFlags(&ctx->cap_main, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&ctx->fork, cudaEventDisableTiming) != cudaSuccess)

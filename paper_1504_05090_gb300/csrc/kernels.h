@@ -138,6 +138,13 @@ cudaError_t launch_gj_inverse(double* A, long long sA, int n, int batch, double*
 cudaError_t launch_qrp_cluster(double* Xt, long long sX, double* Qt, long long sQ, double* D,
                                long long sD, double* Rtil, long long sR, double* vnorm, int n,
                                int batch, int* status, cudaStream_t st);
+// The same QR with the matrix in shared memory (k_qr_smem.cu), `cs` CTAs per
+// matrix: 1 (n <= 144), 4 or 8 (64 < n <= 144).  qr_smem_ctas gives the choice
+// for a context of `chains` chains (0: n is left to another kernel).
+int qr_smem_ctas(int n, int chains, int nsm);
+cudaError_t launch_qr_smem(int cs, double* Xt, long long sX, double* Qt, long long sQ, double* D,
+                           long long sD, double* Rtil, long long sR, int n, int batch, int* status,
+                           cudaStream_t st);
 // Blocked Householder QR with panel-wise pivoting (k_qr_blocked.cu): the same
 // inputs and outputs as launch_qrp_cluster (X^T in, Q^T, D, Rtil out); the
 // remaining columns are sorted by norm at every panel of 32 and pivoted within
