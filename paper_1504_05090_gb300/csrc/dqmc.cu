@@ -430,12 +430,22 @@ int form_mid(dqmc_ctx* ctx, Group& g, int j0, long long es, int batch, double* o
   return DQMC_OK;
 }
 
+// Ainv = A^{-1} of `batch` middle matrices of the group (A may be
+// overwritten), `conc` of all groups' matrices in flight at once; pair:
+// eliminate in float pairs.
+cudaError_t invert(dqmc_ctx* ctx, Group& g, double* A, double* Ainv, int batch, long long conc,
+                   double* logabs, bool pair) {
+  const int cs = gj_smem_ctas(g.N, conc, ctx->nsm, pair);
+  if (cs > 0)
+    return launch_gj_smem(cs, A, g.nn(), Ainv, g.nn(), g.N, batch, logabs, ctx->d_status, g.st, pair);
+  return launch_gj_cluster(A, g.nn(), Ainv, g.nn(), g.N, batch, logabs, ctx->d_status, g.st, pair);
+}
+
 // G64 = U_L Db_L^{-1} Mid^{-1} Db_R^{-1} U_R^T at stack entry j of every chain.
 int recompute(dqmc_ctx* ctx, Group& g, int j) {
   DQ_RET(form_mid(ctx, g, j, g.sstride(), g.C, g.X));
   DQ_CLASS(ctx, kTInverse);
-  DQ_LAUNCH(ctx, launch_gj_cluster(g.X, g.nn(), g.G64, g.nn(), g.N, g.C, nullptr, ctx->d_status,
-                                   g.st));
+  DQ_LAUNCH(ctx, invert(ctx, g, g.X, g.G64, g.C, ctx->total, nullptr, false));
   // U_L (Db_L^{-1} Mid^{-1}): Mid^{-1} grows like Db_L along its rows, so the
   // scale is folded into them (Db_L^{-1} Mid^{-1} Db_R^{-1} is O(|G|)).
   GemmArgs m = gemm0(g.N);
@@ -601,8 +611,7 @@ int all_points_w1(dqmc_ctx* ctx, Group& g, bool pair) {
   const int batch = g.C * (g.nc + 1);
   DQ_RET(form_mid(ctx, g, 0, g.nn(), batch, g.Mid));
   DQ_CLASS(ctx, pair ? kTInversePair : kTInverse);
-  DQ_LAUNCH(ctx, launch_gj_cluster(g.Mid, g.nn(), g.A2, g.nn(), g.N, batch, pair ? nullptr : g.logabs,
-                                   ctx->d_status, g.st, pair));
+  DQ_LAUNCH(ctx, invert(ctx, g, g.Mid, g.A2, batch, batch, pair ? nullptr : g.logabs, pair));
   GemmArgs m = gemm0(g.N);
   m.A = g.LU; m.sA = g.nn(); m.tA = 1;
   m.ks = g.LD; m.sks = g.N; m.ks_mode = 2;

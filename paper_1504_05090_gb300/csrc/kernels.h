@@ -167,6 +167,12 @@ int qr_blocked_launches(int n, int batch, int oz_batch);
 // logabs stay FP64).
 cudaError_t launch_gj_cluster(double* A, long long sA, double* Ainv, long long sI, int n, int batch,
                               double* logabs, int* status, cudaStream_t st, bool pair = false);
+// The same inverse with the matrix in shared memory (k_gj_smem.cu; A is only
+// read), `cs` CTAs per matrix: 1 (n <= 144), 4 or 8.  gj_smem_ctas gives the
+// choice for `conc` matrices in flight (0: launch_gj_cluster).
+int gj_smem_ctas(int n, long long conc, int nsm, bool pair);
+cudaError_t launch_gj_smem(int cs, const double* A, long long sA, double* Ainv, long long sI, int n,
+                           int batch, double* logabs, int* status, cudaStream_t st, bool pair);
 cudaError_t launch_set_identity(double* M, long long sM, double* D, long long sD, int n, int batch,
                                 cudaStream_t st);
 template <typename T>
