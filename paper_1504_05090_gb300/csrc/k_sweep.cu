@@ -40,22 +40,20 @@ __global__ void k_init_field(int8_t* field, int C, int L, int N, int chain0, uin
 }
 
 // ---------------------------------------------------------------------------
-// Metropolis pass over the N sites of one slice, one CTA per chain, one
-// thread per row/column index j.  G (row-major, working precision) stays in
-// global memory (L2-resident); accepted flips are buffered as column vectors
-// U[m] and row vectors V[m] in shared memory, G_cur = G + sum_m U[m] V[m]^T,
-// and folded into G every k accepts (delayed rank-k update).  The diagonal of
-// G_cur is tracked in shared memory so that a rejected proposal costs O(1).
-// The accept/reject decision is taken in FP64 by lane 0 of every warp and
-// broadcast with a shuffle, so all threads agree without a barrier.
+// Metropolis pass over the N sites of one slice, one cluster of cs CTAs per
+// chain.  G (row-major, working precision) stays in global memory
+// (L2-resident); accepted flips are buffered as column vectors U[m] and row
+// vectors V[m] in shared memory, G_cur = G + sum_m U[m] V[m]^T, and folded into
+// G every k accepts (delayed rank-k update).  The diagonal of G_cur is tracked
+// in shared memory so that a rejected proposal costs O(1).  Between two accepted
+// flips the diagonal does not change, so the 32 lanes of every warp decide 32
+// sites at once and take the first accepted one; all warps agree without a
+// barrier.
 // ---------------------------------------------------------------------------
 // Working-precision helpers.
 __device__ __forceinline__ float to_f32(float x) { return x; }
 __device__ __forceinline__ float to_f32(double x) { return static_cast<float>(x); }
 __device__ __forceinline__ float to_f32(df32 x) { return x.hi + x.lo; }
-__device__ __forceinline__ float shfl0(float x) { return __shfl_sync(0xFFFFFFFFu, x, 0); }
-__device__ __forceinline__ double shfl0(double x) { return __shfl_sync(0xFFFFFFFFu, x, 0); }
-__device__ __forceinline__ df32 shfl0(df32 x) { return df32(shfl0(x.hi), shfl0(x.lo)); }
 
 // Sherman-Morrison coefficient -Delta_up / R_up in the working precision:
 // FP32 for float, FP64 for double, and a float reciprocal refined by one
@@ -77,21 +75,103 @@ __device__ __forceinline__ df32 sm_coef(const MetroArgs& a, int s, df32 g) {
   return -(du * y);
 }
 
-// Column j of G, rows ra .. rb-1: G += U V^T over the cnt pending updates.
-// MC = kMaxDelay keeps all of column j of V in registers for the whole flush;
-// a smaller MC reloads it in chunks of MC per row batch (fewer registers, the
-// same additions in the same order).
-template <typename T, int RB = 8, int MC = kMaxDelay>
-__device__ __forceinline__ void delayed_flush(T* G, const T* U, const T* V, int cnt, int N, int NP,
-                                              int j, int ra, int rb) {
-  if (j >= N) return;
-  T v[MC];
-  if constexpr (MC == kMaxDelay) {
-#pragma unroll
-    for (int m = 0; m < kMaxDelay; ++m) v[m] = (m < cnt) ? V[m * NP + j] : T(0);
+// Float pairs, two at a time: a 64-bit register pair holds the high (or low)
+// words of two neighbouring rows, and one packed FP32 instruction works on
+// both.  The packed forms run at the lane rate of the scalar ones (measured
+// 117 against 108 lanes per clock and SM) with half the instructions to issue;
+// every lane rounds as the scalar instruction does, so the sums are the same
+// bit for bit.
+__device__ __forceinline__ uint64_t pk_pack(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void pk_unpack(uint64_t x, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x));
+}
+__device__ __forceinline__ uint64_t pk_mul(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t pk_add(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t pk_sub(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t pk_fma(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+// Two ProdSum<df32> side by side: the same twelve operations per term; the
+// high product is formed negated (-uh vh), which is exact.
+struct ProdSum2 {
+  uint64_t hi, lo;
+  __device__ __forceinline__ ProdSum2() : hi(0ull), lo(0ull) {}
+  // vh, vl: splats of the second factor's words, nvh: of its negated high word;
+  // kSwap: the second factor comes first in the product's error terms
+  template <bool kSwap = false>
+  __device__ __forceinline__ void add(uint64_t uh, uint64_t ul, uint64_t vh, uint64_t vl, uint64_t nvh) {
+    const uint64_t np = pk_mul(uh, nvh);
+    uint64_t e = pk_fma(uh, vh, np);
+    e = kSwap ? pk_fma(ul, vh, e) : pk_fma(uh, vl, e);
+    e = kSwap ? pk_fma(uh, vl, e) : pk_fma(ul, vh, e);
+    const uint64_t t = pk_sub(hi, np);
+    const uint64_t bb = pk_sub(t, hi);
+    const uint64_t x = pk_sub(hi, pk_sub(t, bb));
+    const uint64_t y = pk_add(np, bb);  // -(p - bb)
+    lo = pk_add(lo, pk_add(pk_sub(x, y), e));
+    hi = t;
   }
-  // Rows in batches of RB, the next batch loaded while the current one is
-  // computed, so two batches of L2 loads are in flight per thread.
+  __device__ __forceinline__ void get(df32& a, df32& b) const {
+    float h0, h1, l0, l1;
+    pk_unpack(hi, h0, h1);
+    pk_unpack(lo, l0, l1);
+    a = df_fast_two_sum(h0, l0);
+    b = df_fast_two_sum(h1, l1);
+  }
+};
+
+// U (or V) of the pending updates: [k][NP] numbers, or for float pairs [k][NP]
+// high words followed by [k][NP] low words, so that neighbouring entries load
+// as one packed operand.
+template <typename T>
+struct UStore {
+  T* u;
+  int NP;
+  __device__ __forceinline__ UStore(T* base, int, int np) : u(base), NP(np) {}
+  __device__ __forceinline__ T get(int m, int j) const { return u[m * NP + j]; }
+  __device__ __forceinline__ void set(int m, int j, T x) const { u[m * NP + j] = x; }
+};
+template <>
+struct UStore<df32> {
+  float *h, *l;
+  int NP;
+  __device__ __forceinline__ UStore(df32* base, int k, int np)
+      : h(reinterpret_cast<float*>(base)), l(h + k * np), NP(np) {}
+  __device__ __forceinline__ df32 get(int m, int j) const { return df32(h[m * NP + j], l[m * NP + j]); }
+  __device__ __forceinline__ void set(int m, int j, df32 x) const {
+    h[m * NP + j] = x.hi;
+    l[m * NP + j] = x.lo;
+  }
+};
+
+// Column j of G, rows ra .. rb-1 (both multiples of 4): G += U V^T over the cnt
+// pending updates, eight rows at a time, the next eight loaded while the
+// current ones are computed.  Column j of V is read in chunks of MC updates
+// per row batch (the same additions in the same order for any MC).
+template <typename T, int MC>
+__device__ __forceinline__ void delayed_flush(T* G, const UStore<T>& U, const UStore<T>& V, int cnt, int N,
+                                              int NP, int j, int ra, int rb) {
+  constexpr int RB = 8;
+  if (j >= N) return;
   T cur[RB], nxt[RB];
 #pragma unroll
   for (int q = 0; q < RB; ++q) cur[q] = (ra + q < rb) ? G[static_cast<size_t>(ra + q) * N + j] : T(0);
@@ -100,40 +180,81 @@ __device__ __forceinline__ void delayed_flush(T* G, const T* U, const T* V, int 
 #pragma unroll
     for (int q = 0; q < RB; ++q)
       nxt[q] = (r1 + q < rb) ? G[static_cast<size_t>(r1 + q) * N + j] : T(0);
-    ProdSum<T> acc[RB];
-    for (int m0 = 0; m0 < cnt; m0 += MC) {
-      if constexpr (MC != kMaxDelay) {
+    if constexpr (std::is_same<T, df32>::value) {
+      // 2 x 16-byte loads of U and twelve packed instructions per update and
+      // four rows; bound by the FP32 pipe (64 packed lanes per clock and SM)
+      ProdSum2 acc[RB / 2];
+      // a chunk of MC updates without a branch inside, so that its loads are
+      // issued ahead of its arithmetic; then the rest one by one
+      auto chunk = [&](auto width, int m0) {
+        constexpr int W = decltype(width)::value;
+        uint64_t vh[W], vl[W], nvh[W];
 #pragma unroll
-        for (int mm = 0; mm < MC; ++mm) v[mm] = (m0 + mm < cnt) ? V[(m0 + mm) * NP + j] : T(0);
-      }
-      if constexpr (std::is_same<T, df32>::value && RB % 2 == 0) {
-        // two rows of U per 16-byte load when the row pair is 16-byte aligned
-        // (r0 even: U rows of NP entries start 16-byte aligned); the sums of
-        // each row see the same additions in the same order either way
-        if ((r0 & 1) == 0) {
-#pragma unroll
-          for (int q = 0; q < RB; q += 2) {
-#pragma unroll
-            for (int mm = 0; mm < MC; ++mm)
-              if (m0 + mm < cnt) {
-                const float4 u2 = *reinterpret_cast<const float4*>(U + (m0 + mm) * NP + r0 + q);
-                acc[q].add(df32(u2.x, u2.y), v[mm]);
-                acc[q + 1].add(df32(u2.z, u2.w), v[mm]);
-              }
-          }
-          continue;
+        for (int mm = 0; mm < W; ++mm) {
+          const df32 v = V.get(m0 + mm, j);
+          vh[mm] = pk_pack(v.hi, v.hi);
+          vl[mm] = pk_pack(v.lo, v.lo);
+          nvh[mm] = pk_pack(-v.hi, -v.hi);
         }
-      }
 #pragma unroll
-      for (int q = 0; q < RB; ++q) {
+        for (int q = 0; q < RB; q += 4) {
+          ulonglong2 uh[W], ul[W];
 #pragma unroll
-        for (int mm = 0; mm < MC; ++mm)
-          if (m0 + mm < cnt) acc[q].add(U[(m0 + mm) * NP + r0 + q], v[mm]);
+          for (int mm = 0; mm < W; ++mm) {
+            uh[mm] = *reinterpret_cast<const ulonglong2*>(U.h + (m0 + mm) * NP + r0 + q);
+            ul[mm] = *reinterpret_cast<const ulonglong2*>(U.l + (m0 + mm) * NP + r0 + q);
+          }
+#pragma unroll
+          for (int mm = 0; mm < W; ++mm) {
+            acc[q / 2].add(uh[mm].x, ul[mm].x, vh[mm], vl[mm], nvh[mm]);
+            acc[q / 2 + 1].add(uh[mm].y, ul[mm].y, vh[mm], vl[mm], nvh[mm]);
+          }
+        }
+      };
+      int m0 = 0;
+      for (; m0 + MC <= cnt; m0 += MC) chunk(std::integral_constant<int, MC>(), m0);
+      for (; m0 < cnt; ++m0) chunk(std::integral_constant<int, 1>(), m0);
+#pragma unroll
+      for (int q = 0; q < RB; q += 2) {
+        df32 s0, s1;
+        acc[q / 2].get(s0, s1);
+        if (r0 + q < rb) G[static_cast<size_t>(r0 + q) * N + j] = cur[q] + s0;
+        if (r0 + q + 1 < rb) G[static_cast<size_t>(r0 + q + 1) * N + j] = cur[q + 1] + s1;
       }
+    } else {
+      ProdSum<T> acc[RB];
+      auto chunk = [&](auto width, int m0) {
+        constexpr int W = decltype(width)::value;
+        T v[W];
+#pragma unroll
+        for (int mm = 0; mm < W; ++mm) v[mm] = V.get(m0 + mm, j);
+        if constexpr (std::is_same<T, float>::value) {  // four rows of U per 16-byte load
+#pragma unroll
+          for (int q = 0; q < RB; q += 4) {
+#pragma unroll
+            for (int mm = 0; mm < W; ++mm) {
+              const float4 u = *reinterpret_cast<const float4*>(U.u + (m0 + mm) * NP + r0 + q);
+              acc[q].add(u.x, v[mm]);
+              acc[q + 1].add(u.y, v[mm]);
+              acc[q + 2].add(u.z, v[mm]);
+              acc[q + 3].add(u.w, v[mm]);
+            }
+          }
+        } else {
+#pragma unroll
+          for (int q = 0; q < RB; ++q) {
+#pragma unroll
+            for (int mm = 0; mm < W; ++mm) acc[q].add(U.u[(m0 + mm) * NP + r0 + q], v[mm]);
+          }
+        }
+      };
+      int m0 = 0;
+      for (; m0 + MC <= cnt; m0 += MC) chunk(std::integral_constant<int, MC>(), m0);
+      for (; m0 < cnt; ++m0) chunk(std::integral_constant<int, 1>(), m0);
+#pragma unroll
+      for (int q = 0; q < RB; ++q)
+        if (r0 + q < rb) G[static_cast<size_t>(r0 + q) * N + j] = cur[q] + acc[q].get();
     }
-#pragma unroll
-    for (int q = 0; q < RB; ++q)
-      if (r0 + q < rb) G[static_cast<size_t>(r0 + q) * N + j] = cur[q] + acc[q].get();
 #pragma unroll
     for (int q = 0; q < RB; ++q) cur[q] = nxt[q];
   }
@@ -158,21 +279,26 @@ __device__ __forceinline__ unsigned long long global_ns() {
 
 // `broken` (shared) is set once a wait gave up; later barriers of the launch
 // then only synchronise the CTA.
+// kGlobal: G in global memory is ordered too (a flush); otherwise only the
+// shared memory written to the peers.
+template <bool kGlobal>
 __device__ __forceinline__ void peer_barrier(uint64_t* bars, int cs, int rank, int& phase,
                                              int* status, int* broken) {
   __syncthreads();
-  if (threadIdx.x == 0 && !*broken) {
-    __threadfence();
-    const uint32_t local = static_cast<uint32_t>(__cvta_generic_to_shared(bars + (phase & 1)));
-    for (int r = 0; r < cs; ++r) {
-      if (r == rank) continue;
-      uint32_t remote;
-      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(r));
-      asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(remote)
-                   : "memory");
-    }
+  // thread r arrives at peer r (one after the other they would wait for each
+  // other's release)
+  const bool ok = !*broken;
+  const uint32_t local = static_cast<uint32_t>(__cvta_generic_to_shared(bars + (phase & 1)));
+  if (static_cast<int>(threadIdx.x) < cs && static_cast<int>(threadIdx.x) != rank && ok) {
+    if (kGlobal) __threadfence();
+    uint32_t remote;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(threadIdx.x));
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(remote)
+                 : "memory");
+  }
+  if (threadIdx.x == 0 && ok) {
     uint32_t done = 0;
-    const unsigned long long t0 = global_ns();
+    unsigned long long t0 = 0;  // read only once a wait gets long (the timer is slow)
     for (long long it = 0; it < kPeerWaitPolls && !done; ++it) {
       asm volatile(
           "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
@@ -180,58 +306,82 @@ __device__ __forceinline__ void peer_barrier(uint64_t* bars, int cs, int rank, i
           : "=r"(done)
           : "r"(local), "r"((phase >> 1) & 1)
           : "memory");
-      if (!done && (it & 255) == 255 && global_ns() - t0 > kPeerWaitNs) break;
+      if (!done && (it & 255) == 255) {
+        const unsigned long long now = global_ns();
+        if (t0 == 0) t0 = now;
+        if (now - t0 > kPeerWaitNs) break;
+      }
     }
     if (!done) {
       atomicExch(status, kDevTimeout);
       *broken = 1;
     }
-    __threadfence();
+    if (kGlobal) __threadfence();
   }
   ++phase;
   __syncthreads();
 }
 
-// Threads per column of G: two for float pairs (one computes the column and
-// one the row correction of an accepted flip, and they split the rows of the
-// flush), one otherwise.
 // Columns of G staged in shared memory per window of sites (k_metropolis).
 constexpr int kWin = 32;
+constexpr int kRing = 8;  // rows of G asked for ahead
 
-// Pending updates per register chunk of the flush: all of them for one
-// thread per column; eight for float pairs, whose two threads per column
-// each fold eight rows at a time (more independent sums in flight at the
-// 128-register limit of 512 threads).
+// Pending updates per register chunk of the flush: as many as 128 registers
+// per thread (512 threads) allow beside the eight rows in flight.
 template <typename T>
 constexpr int kFlushMC() {
-  return std::is_same<T, df32>::value ? 8 : kMaxDelay;
+  return std::is_same<T, float>::value ? 16 : std::is_same<T, df32>::value ? 4 : 8;
 }
 
-template <typename T>
-constexpr int metro_halves() {
-  return std::is_same<T, df32>::value ? 2 : 1;
-}
+constexpr int kHalves = 2;
+constexpr int kMetroThreads = kHalves * kMaxN;  // most threads per CTA besides the scalar warp
 
+// H = 2 threads per column (4 and 8 were measured: never faster, and up to
+// twice slower with many small chains); both share the rows of a flush.  Of an
+// accepted flip, half of the working threads (role 0) correct the column G e_i
+// for the pending updates, the other half (role 1) the row e_i^T G, one column
+// each; float pairs take two columns per thread with packed instructions, so
+// that half of the warps have no part in a flip: they wait at the CTA's
+// barrier for the next flush, and the flips synchronise the others only.  In
+// FP32, where a flip is little more than its barriers, one thread does both for
+// its column and the flip needs one barrier instead of two.  One warp forms the
+// Sherman-Morrison coefficient of the flip: a chain of dependent operations
+// that, repeated by every warp, took more of the FP64 pipe than the
+// corrections.  In FP64 it is a warp of its own (kScalarWarp); for float pairs,
+// whose flush needs the registers that a 17th warp would cost, one of the idle
+// warps (if there is one).
+//
 // Thread-block cluster of cs CTAs per chain (cs = 1: one CTA).  Every CTA
-// takes the same site decisions and builds the same U, V from the same data
-// (identical instruction streams, so identical results); in a flush each CTA
-// adds U V^T to its own block of N / cs rows of G.  Two peer barriers bracket
-// every flush: no CTA overwrites rows that a peer may still read for the
-// sites before the flush, and every CTA reads the new rows after it.
+// takes the same site decisions from the same data (identical instruction
+// streams, so identical results); in a flush each CTA adds U V^T to its own
+// block of rows of G.  Two peer barriers bracket every flush: no CTA
+// overwrites rows that a peer may still read for the sites before the flush,
+// and every CTA reads the new rows after it.  U and V are formed by every CTA
+// for itself, or, in FP64 from N = 128 on (kSplitN), each CTA corrects only its
+// share of the columns and sends the entries to its peers: the corrections are
+// then a quarter of the FP64 work of a pass instead of a copy of it on every
+// SM, for one more peer barrier per accepted flip.
+constexpr int kSplitN = 128;
+
 template <typename T>
-__global__ void __launch_bounds__(256 * metro_halves<T>()) k_metropolis(T* Gall, int8_t* fieldall,
-                                                                      MetroArgs a) {
-  constexpr int kH = metro_halves<T>();
+constexpr bool kScalarWarp() {
+  return std::is_same<T, double>::value;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kMetroThreads + (kScalarWarp<T>() ? 32 : 0)) k_metropolis(T* Gall, int8_t* fieldall, MetroArgs a) {
   const int cs = a.cs;
   const int c = blockIdx.x / cs;
   const int rank = blockIdx.x - c * cs;  // cluster rank (the cluster spans blockIdx.x)
   const int N = a.N;
-  const int NP = blockDim.x / kH;                // columns (N rounded up to a warp)
-  const int h = (kH == 2 && static_cast<int>(threadIdx.x) >= NP) ? 1 : 0;
-  // rows of G this thread folds the delayed updates into: the CTA's block of
-  // N / cs rows, split between the two halves when kH = 2
-  const int ra0 = (rank * N) / cs, rb0 = ((rank + 1) * N) / cs, rmid = ra0 + (rb0 - ra0 + 1) / 2;
-  const int ra = (kH == 2 && h) ? rmid : ra0, rb = (kH == 2 && !h) ? rmid : rb0;
+  constexpr int H = kHalves;
+  const int NP = (blockDim.x - (kScalarWarp<T>() ? 32 : 0)) / H;  // columns (N rounded up to a warp)
+  const int h = threadIdx.x / NP;        // H: the scalar warp
+  // rows of G this thread folds the delayed updates into, in units of four:
+  // the CTA's block, split between its H thread groups
+  const int n4 = N >> 2, part = rank * H + h, parts = cs * H;
+  const int ra = 4 * ((part * n4) / parts), rb = (h < H) ? 4 * (((part + 1) * n4) / parts) : 0;
+  __shared__ T coef_sh;
   __shared__ uint64_t xbar[2];
   __shared__ int xbroken;
   int xphase = 0;
@@ -250,19 +400,22 @@ __global__ void __launch_bounds__(256 * metro_halves<T>()) k_metropolis(T* Gall,
   }
   const int j = threadIdx.x - h * NP;  // column of this thread
   const int lane = threadIdx.x & 31;
-  const bool act = j < N;
+  const bool act = h < H && j < N;
   T* G = Gall + static_cast<size_t>(c) * N * N;
   int8_t* s_l = fieldall + (static_cast<size_t>(c) * a.L + a.l0) * N;
 
   extern __shared__ __align__(16) unsigned char sm_raw[];
   double* uu = reinterpret_cast<double*>(sm_raw);  // [NP] proposal uniforms
   float* uuf = reinterpret_cast<float*>(uu + NP);   // [NP] the same, rounded to float
-  T* U = reinterpret_cast<T*>(uuf + NP);            // [k][NP]
-  T* V = U + a.k * NP;                              // [k][NP]
-  T* d = V + a.k * NP;                              // [NP] diag of G_cur
+  T* Ubase = reinterpret_cast<T*>(uuf + NP);        // [k][NP], see UStore
+  const UStore<T> U(Ubase, a.k, NP);
+  T* Vbase = Ubase + a.k * NP;                      // [k][NP]
+  const UStore<T> V(Vbase, a.k, NP);
+  T* d = Vbase + a.k * NP;                          // [NP] diag of G_cur
   float* df = reinterpret_cast<float*>(d + NP);     // [NP] diag of G_cur, rounded to float
   int* ss = reinterpret_cast<int*>(df + NP);        // [NP] field of the slice
-  T* cw = reinterpret_cast<T*>(ss + NP);            // [kWin][NP + 1] window of columns of G
+  T* ring = reinterpret_cast<T*>(ss + NP);          // [kRing][NP] rows of G to come (FP32)
+  T* cw = ring + (std::is_same<T, float>::value ? kRing * NP : 0);  // [kWin][NP + 1] window of columns of G
 
   const uint32_t sweep = *a.sweep_ctr;
   if (act && h == 0) {
@@ -283,155 +436,347 @@ __global__ void __launch_bounds__(256 * metro_halves<T>()) k_metropolis(T* Gall,
   // loaded with whole-row segments (a column of the row-major G would take one
   // memory transaction per row), reloaded every kWin sites and after a flush.
   const int ldw = NP + 1;  // odd stride in 8-byte words: conflict-free transposed stores
-  auto load_window = [&](int wb) {
+  auto load_window = [&](int wb, int nthr) {
     constexpr int kU = 8;
     const int tot = N * kWin;
-    for (int e0 = threadIdx.x; e0 < tot; e0 += kU * blockDim.x) {
+    for (int e0 = threadIdx.x; e0 < tot; e0 += kU * nthr) {
       T t[kU];
 #pragma unroll
       for (int u = 0; u < kU; ++u) {
-        const int e = e0 + u * blockDim.x, r = e / kWin, c = e - r * kWin;
+        const int e = e0 + u * nthr, r = e / kWin, c = e - r * kWin;
         t[u] = (e < tot && wb + c < N) ? G[static_cast<size_t>(r) * N + wb + c] : T(0);
       }
 #pragma unroll
       for (int u = 0; u < kU; ++u) {
-        const int e = e0 + u * blockDim.x, r = e / kWin, c = e - r * kWin;
+        const int e = e0 + u * nthr, r = e / kWin, c = e - r * kWin;
         if (e < tot) cw[c * ldw + r] = t[u];
       }
     }
   };
   int wb = 0;
-  load_window(0);
+  load_window(0, blockDim.x);
   __syncthreads();
-  // Row i of G for the next kPre sites, loaded ahead into registers (rows
-  // are contiguous; a flush rewrites G, after which the window is reloaded).
-  // With two threads per column only the row half uses it.
-  constexpr int kPre = 4;
-  T pr[kPre];
-  auto ld_r = [&](int q) -> T {
-    return (act && q < N && (kH == 1 || h == 1)) ? G[static_cast<size_t>(q) * N + j] : T(0);
+  // The entry of U (role 0) or V (role 1) that this thread forms of an accepted
+  // flip: its own column cj, or with a split correction one of the CTA's share
+  // (the first 2 ns threads); float pairs: two neighbouring columns cj, cj + 1
+  // with packed instructions.  role < 0: none.
+  constexpr bool kPair = std::is_same<T, df32>::value;
+  constexpr bool kBoth = std::is_same<T, float>::value;  // role 2: column and row
+  const bool split = std::is_same<T, double>::value && cs > 1 && N >= kSplitN;
+  int role = (h < 2 && act) ? h : -1, cj = j;
+  // kPair: warps 0 .. pw-1 role 0, pw .. 2 pw-1 role 1, the next (if there is
+  // one) the coefficient; all others only flush
+  const int warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5, pw = (NP / 2 + 31) >> 5;
+  const int nact = kPair ? 32 * min(nwarp, 2 * pw + 1) : kBoth ? NP : static_cast<int>(blockDim.x);
+  if (kBoth) role = (h == 0 && act) ? 2 : -1;
+  if (kPair) {
+    role = warp < pw ? 0 : warp < 2 * pw ? 1 : -1;
+    cj = 2 * (static_cast<int>(threadIdx.x) - 32 * pw * max(role, 0));
+    if (cj >= N) role = -1;
+  }
+  const int coef_thread = kScalarWarp<T>() ? H * NP : (nwarp > 2 * pw ? 64 * pw : 32 * pw);
+  if (split) {
+    const int s0 = (rank * N) / cs, ns = ((rank + 1) * N) / cs - s0;
+    role = static_cast<int>(threadIdx.x) / ns;
+    cj = s0 + static_cast<int>(threadIdx.x) - role * ns;
+    if (role > 1) role = -1;
+  }
+  // Rows of G of the sites to come, asked for ahead by the threads of role 1
+  // (or 2), each for its own columns.  Float pairs and FP64 keep the kPre rows
+  // after the last accepted site in registers; in FP32, where an L2 access takes
+  // about as long as a flip, cp.async brings rows kRing sites ahead into a ring
+  // in shared memory (for the other types the ring's bookkeeping cost more than
+  // the wait: 686 against 663 us per slice, 16 x 16 in float pairs; FP32 8 x 8
+  // with it 48 instead of 52 us).  A flush rewrites G, after which the rows are
+  // asked for again.
+  struct Entry {
+    T x[kPair ? 2 : 1];
   };
+  auto ld_row = [&](int q) -> Entry {
+    Entry e;
+    const T* src = G + static_cast<size_t>(q) * N + cj;
+    if constexpr (kPair) {
+      const float4 f = *reinterpret_cast<const float4*>(src);
+      e.x[0] = df32(f.x, f.y);
+      e.x[1] = df32(f.z, f.w);
+    } else {
+      e.x[0] = *src;
+    }
+    return e;
+  };
+  constexpr int kPre = 2;
+  Entry pr[kPre];
+  // first row in pr; for the ring: the last group of copies holds rows pbase ..
+  // rq-1
+  int pbase = 0, rq = 0;
+  auto prefetch = [&](int q0) {
+    if (role < 1) return;
+    if constexpr (kBoth) {
+      pbase = max(rq, q0);
+      const int qe = min(q0 + kRing, N);
+      for (rq = pbase; rq < qe; ++rq)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(static_cast<uint32_t>(
+                         __cvta_generic_to_shared(ring + (rq % kRing) * NP + cj))),
+                     "l"(G + static_cast<size_t>(rq) * N + cj)
+                     : "memory");
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    } else {
+      pbase = q0;
 #pragma unroll
-  for (int q = 0; q < kPre; ++q) pr[q] = ld_r(q);
+      for (int q = 0; q < kPre; ++q)
+        if (q0 + q < N) pr[q] = ld_row(q0 + q);
+    }
+  };
+  auto row_entry = [&](int i) -> Entry {  // the own entries of row i
+    if constexpr (kBoth) {
+      if (i >= rq) return ld_row(i);  // further ahead than the ring
+      if (i >= pbase)
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+      else
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+      Entry e;
+      e.x[0] = ring[(i % kRing) * NP + cj];
+      return e;
+    } else {
+      return i == pbase ? pr[0] : i == pbase + 1 ? pr[1] : ld_row(i);
+    }
+  };
+  prefetch(0);
   int cnt = 0;
   unsigned naccept = 0;
-  // The field is written back after the slice: a peer CTA of the cluster may
-  // still be reading the slice's initial field when this one accepts a flip.
-  bool flip = false;
-  for (int i = 0; i < N; ++i) {
-    if (i == wb + kWin) {  // every warp is past site i - 1
+  // pending updates of a flush and the first site of the next window (-1: the
+  // slice ends), for the warps that take no part in the flips
+  __shared__ int flush_sh[2];
+  // barrier of the warps that work on the flips
+  auto sync_act = [&]() {
+    if constexpr (kPair || kBoth)
+      asm volatile("bar.sync 1, %0;" ::"r"(nact) : "memory");
+    else
       __syncthreads();
-      wb = i;
-      load_window(wb);
-      __syncthreads();
-    }
-    // kH == 2: colv is G[j][i] for h = 0 and rowv G[i][j] for h = 1
-    const T colv = act ? cw[(i - wb) * ldw + j] : T(0);
-    const T rowv = pr[0];
-#pragma unroll
-    for (int q = 0; q + 1 < kPre; ++q) pr[q] = pr[q + 1];
-    pr[kPre - 1] = ld_r(i + kPre);
-    // Decision u < R_up R_dn with R_up = 1 + D_up (1 - G_ii), R_dn = 1 + D_dn G_ii
-    // (G_dn,ii = 1 - G_up,ii).  Lane 0 of every warp takes it in FP32 unless u
-    // lies within 1e-4 of R, where it is retaken in FP64; all warps agree
-    // without a barrier.
-    int acc_i = 0;
-    T coef = T(0);
-    if (lane == 0) {
-      const int s = ss[i];
-      const float gf = df[i];
-      const float duf = s > 0 ? a.em2h : a.ep2h, ddf = s > 0 ? a.ep2h : a.em2h;
-      const float Rf = fmaf(duf, 1.0f - gf, 1.0f) * fmaf(ddf, gf, 1.0f);
-      const float uf = uuf[i];
-      if (uf < Rf * 0.9999f) {
-        acc_i = 1;
-      } else if (!(uf > Rf * 1.0001f)) {
-        const double g = static_cast<double>(d[i]);
-        const double du = s > 0 ? a.em2 : a.ep2, dd = s > 0 ? a.ep2 : a.em2;
-        acc_i = uu[i] < fma(du, 1.0 - g, 1.0) * fma(dd, g, 1.0);
-      }
-      if (acc_i) coef = sm_coef(a, s, d[i]);
-    }
-    acc_i = __shfl_sync(0xFFFFFFFFu, acc_i, 0);
-    if (acc_i) {
-      coef = shfl0(coef);
-      ++naccept;
-      if constexpr (kH == 1) {
-        if (act) {
-          ProdSum<T> sc, sr;
-          for (int m = 0; m < cnt; ++m) {
-            sc.add(U[m * NP + j], V[m * NP + i]);
-            sr.add(U[m * NP + i], V[m * NP + j]);
-          }
-          const T gc = colv + sc.get(), gr = rowv + sr.get();
-          const T uj = coef * ((j == i ? T(1) : T(0)) - gc);
-          U[cnt * NP + j] = uj;
-          V[cnt * NP + j] = gr;
-          // Only the diagonal of sites still to come (j > i) is updated.  Warps
-          // pass rejected sites without a barrier, so a slower warp may still be
-          // deciding an earlier site j <= i: its d[j], df[j] (dead for the rest
-          // of the slice) must keep the value every other warp decided with.
-          if (j > i) {
-            const T dj = d[j] + uj * gr;
-            d[j] = dj;
-            df[j] = to_f32(dj);
-          } else if (j == i) {
-            flip = true;
+  };
+  int i = 0;
+  do {
+    if (static_cast<int>(threadIdx.x) < nact) {
+      while (i < N && cnt < a.k) {
+        // Decision u < R_up R_dn with R_up = 1 + D_up (1 - G_ii), R_dn = 1 + D_dn G_ii
+        // (G_dn,ii = 1 - G_up,ii) of sites i .. i + 31, one per lane: in FP32 unless
+        // u lies within 1e-4 of R, where it is retaken in FP64.
+        bool acc = false;
+        if (i + lane < N) {
+          const int q = i + lane, s = ss[q];
+          const float gf = df[q];
+          const float duf = s > 0 ? a.em2h : a.ep2h, ddf = s > 0 ? a.ep2h : a.em2h;
+          const float Rf = fmaf(duf, 1.0f - gf, 1.0f) * fmaf(ddf, gf, 1.0f);
+          const float uf = uuf[q];
+          if (uf < Rf * 0.9999f) {
+            acc = true;
+          } else if (!(uf > Rf * 1.0001f)) {
+            const double g = static_cast<double>(d[q]);
+            const double du = s > 0 ? a.em2 : a.ep2, dd = s > 0 ? a.ep2 : a.em2;
+            acc = uu[q] < fma(du, 1.0 - g, 1.0) * fma(dd, g, 1.0);
           }
         }
-      } else {
-        // column correction (h = 0) and row correction (h = 1) of the flip
-        if (act) {
-          ProdSum<T> sa;
-          if (h == 0) {
-            for (int m = 0; m < cnt; ++m) sa.add(U[m * NP + j], V[m * NP + i]);
-            const T gc = colv + sa.get();
-            U[cnt * NP + j] = coef * ((j == i ? T(1) : T(0)) - gc);
+        const unsigned hits = __ballot_sync(0xFFFFFFFFu, acc);
+        if (hits == 0u) {
+          i += 32;
+          continue;
+        }
+        i += __ffs(hits) - 1;  // the next accepted site
+        if (i >= wb + kWin) {  // nobody reads the window between two accepted sites
+          wb = i;
+          load_window(wb, nact);
+          sync_act();
+        }
+        ++naccept;
+        if constexpr (kBoth) {
+          T coef = T(0);
+          if (lane == 0) coef = sm_coef(a, ss[i], d[i]);
+          coef = __shfl_sync(0xFFFFFFFFu, coef, 0);
+          if (role == 2) {
+            ProdSum<T> sc, sr;
+#pragma unroll 4
+            for (int m = 0; m < cnt; ++m) {
+              sc.add(U.get(m, j), V.get(m, i));
+              sr.add(U.get(m, i), V.get(m, j));
+            }
+            const T row = row_entry(i).x[0];
+            const T uj = coef * ((j == i ? T(1) : T(0)) - (cw[(i - wb) * ldw + j] + sc.get()));
+            const T vj = row + sr.get();
+            U.set(cnt, j, uj);
+            V.set(cnt, j, vj);
+            // a slower warp may still be deciding: what it reads of the sites
+            // up to i is left alone, and what it makes of later ones, beyond
+            // the first accepted site i, it does not use
+            if (j > i) {
+              const T dj = d[j] + uj * vj;
+              d[j] = dj;
+              df[j] = to_f32(dj);
+            }
+          }
+          prefetch(i + 1);
+          sync_act();
+          if (threadIdx.x == 0) ss[i] = -ss[i];  // site i is not read again
+          ++cnt;
+          ++i;
+          continue;
+        }
+        if (static_cast<int>(threadIdx.x) == coef_thread) coef_sh = sm_coef(a, ss[i], d[i]);
+        // column (role 0: e_i - G e_i, scaled below) or row (role 1: e_i^T G)
+        // entry of G_cur, four updates' loads at a time ahead of their serial sums
+        Entry w0;  // role 0 of float pairs: the unscaled entries of U
+        if (role >= 0) {
+          // the entry of G, read after the sums
+          auto g_entry = [&]() -> Entry {
+            Entry e;
+            if (role == 0) {
+              e.x[0] = cw[(i - wb) * ldw + cj];
+              if constexpr (kPair) e.x[1] = cw[(i - wb) * ldw + cj + 1];
+            } else {
+              e = row_entry(i);
+            }
+            return e;
+          };
+          int m = 0;
+          if constexpr (kPair) {
+            const UStore<df32>& P = role == 0 ? U : V;  // two entries of the own columns
+            const UStore<df32>& S = role == 0 ? V : U;  // the entry of site i
+            ProdSum2 sa;
+            auto terms = [&](auto width, auto swap) {
+              constexpr int W = decltype(width)::value;
+              uint64_t ph[W], pl[W];
+              df32 sp[W];
+#pragma unroll
+              for (int q = 0; q < W; ++q) {
+                ph[q] = *reinterpret_cast<const uint64_t*>(P.h + (m + q) * NP + cj);
+                pl[q] = *reinterpret_cast<const uint64_t*>(P.l + (m + q) * NP + cj);
+                sp[q] = S.get(m + q, i);
+              }
+#pragma unroll
+              for (int q = 0; q < W; ++q)
+                sa.template add<decltype(swap)::value>(ph[q], pl[q], pk_pack(sp[q].hi, sp[q].hi),
+                                                       pk_pack(sp[q].lo, sp[q].lo), pk_pack(-sp[q].hi, -sp[q].hi));
+            };
+            if (role == 0) {
+              for (; m + 4 <= cnt; m += 4) terms(std::integral_constant<int, 4>(), std::false_type());
+              for (; m < cnt; ++m) terms(std::integral_constant<int, 1>(), std::false_type());
+            } else {
+              for (; m + 4 <= cnt; m += 4) terms(std::integral_constant<int, 4>(), std::true_type());
+              for (; m < cnt; ++m) terms(std::integral_constant<int, 1>(), std::true_type());
+            }
+            df32 s0, s1;
+            sa.get(s0, s1);
+            const Entry g0 = g_entry();
+            if (role == 0) {
+              s0 = (cj == i ? T(1) : T(0)) - (g0.x[0] + s0);
+              s1 = (cj + 1 == i ? T(1) : T(0)) - (g0.x[1] + s1);
+            } else {
+              s0 = g0.x[0] + s0;
+              s1 = g0.x[1] + s1;
+            }
+            if (role == 1) {
+              *reinterpret_cast<uint64_t*>(V.h + cnt * NP + cj) = pk_pack(s0.hi, s1.hi);
+              *reinterpret_cast<uint64_t*>(V.l + cnt * NP + cj) = pk_pack(s0.lo, s1.lo);
+            }
+            w0.x[0] = s0;
+            w0.x[1] = s1;
           } else {
-            for (int m = 0; m < cnt; ++m) sa.add(U[m * NP + i], V[m * NP + j]);
-            V[cnt * NP + j] = rowv + sa.get();
+            ProdSum<T> sa;
+            const int ju = (role == 0) ? cj : i, jv = (role == 0) ? i : cj;
+            for (; m + 4 <= cnt; m += 4) {
+              T u[4], v[4];
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                u[q] = U.get(m + q, ju);
+                v[q] = V.get(m + q, jv);
+              }
+#pragma unroll
+              for (int q = 0; q < 4; ++q) sa.add(u[q], v[q]);
+            }
+            for (; m < cnt; ++m) sa.add(U.get(m, ju), V.get(m, jv));
+            const T gs = g_entry().x[0] + sa.get();
+            const T x = (role == 0) ? (cj == i ? T(1) : T(0)) - gs : gs;
+            if (!split) {
+              (role == 0 ? U : V).set(cnt, cj, x);
+            } else {
+              if constexpr (std::is_same<T, double>::value) {
+                double* dst = (role == 0 ? U.u : V.u) + cnt * NP + cj;
+                cg::cluster_group cl = cg::this_cluster();
+                for (int r = 0; r < cs; ++r) *cl.map_shared_rank(dst, r) = x;
+              }
+            }
           }
         }
-        __syncthreads();
-        // every warp is at site i here, so the diagonal of the sites to come
-        // is updated before anyone decides the next site (barrier below)
-        if (act && h == 0) {
+        prefetch(i + 1);
+        if (split)
+          peer_barrier<false>(xbar, cs, rank, xphase, a.status, &xbroken);
+        else
+          sync_act();
+        // every warp is at site i here, so the diagonal of the sites to come is
+        // updated before anyone decides the next site (barrier below)
+        if constexpr (kPair) {
+          if (role == 0) {
+            const df32 cf = coef_sh;
+            df32 uj[2], dj[2];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+              uj[q] = cf * w0.x[q];
+              dj[q] = d[cj + q] + uj[q] * V.get(cnt, cj + q);
+            }
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+              if (cj + q > i) {
+                d[cj + q] = dj[q];
+                df[cj + q] = to_f32(dj[q]);
+              }
+            *reinterpret_cast<uint64_t*>(U.h + cnt * NP + cj) = pk_pack(uj[0].hi, uj[1].hi);
+            *reinterpret_cast<uint64_t*>(U.l + cnt * NP + cj) = pk_pack(uj[0].lo, uj[1].lo);
+          }
+        } else if (act && h == 0) {
+          const T uj = coef_sh * U.get(cnt, j);
+          U.set(cnt, j, uj);
           if (j > i) {
-            const T dj = d[j] + U[cnt * NP + j] * V[cnt * NP + j];
+            const T dj = d[j] + uj * V.get(cnt, j);
             d[j] = dj;
             df[j] = to_f32(dj);
-          } else if (j == i) {
-            flip = true;
           }
         }
+        if (threadIdx.x == 0) ss[i] = -ss[i];  // site i is not read again
+        ++cnt;
+        ++i;
+        sync_act();
       }
-      __syncthreads();
-      ++cnt;
-      if (cnt == a.k) {
-        if (cs > 1) peer_barrier(xbar, cs, rank, xphase, a.status, &xbroken);
-        delayed_flush<T, 8, kFlushMC<T>()>(G, U, V, cnt, N, NP, j, ra, rb);
-        cnt = 0;
-        if (cs > 1)
-          peer_barrier(xbar, cs, rank, xphase, a.status, &xbroken);
-        else
-          __syncthreads();
-        wb = i + 1;
-        load_window(wb);
-        __syncthreads();
-#pragma unroll
-        for (int q = 0; q < kPre; ++q) pr[q] = ld_r(i + 1 + q);
+      if (threadIdx.x == 0) {
+        flush_sh[0] = cnt;
+        flush_sh[1] = (i < N) ? i : -1;
       }
     }
-  }
-  if (cnt > 0) {
-    if (cs > 1) peer_barrier(xbar, cs, rank, xphase, a.status, &xbroken);
-    delayed_flush<T, 8, kFlushMC<T>()>(G, U, V, cnt, N, NP, j, ra, rb);
-  }
+    // flush, by all warps
+    if (cs > 1)
+      peer_barrier<true>(xbar, cs, rank, xphase, a.status, &xbroken);
+    else
+      __syncthreads();
+    cnt = flush_sh[0];
+    wb = flush_sh[1];
+    if (cnt > 0) delayed_flush<T, kFlushMC<T>()>(G, U, V, cnt, N, NP, j, ra, rb);
+    cnt = 0;
+    if (wb >= 0) {
+      if (cs > 1)
+        peer_barrier<true>(xbar, cs, rank, xphase, a.status, &xbroken);
+      else
+        __syncthreads();
+      load_window(wb, blockDim.x);
+      __syncthreads();
+      rq = wb;
+      prefetch(wb);
+    }
+  } while (wb >= 0);
   // No CTA leaves while a peer may still arrive on its barrier or read the
   // slice's field.
   if (cs > 1) cooperative_groups::this_cluster().sync();
+  // The field is written back after the slice: a peer CTA of the cluster may
+  // still be reading the slice's initial field when this one accepts a flip.
   if (rank == 0) {
-    if (flip) s_l[j] = static_cast<int8_t>(-ss[j]);
+    if (act && h == 0) s_l[j] = static_cast<int8_t>(ss[j]);
     if (threadIdx.x == 0) a.accepted[c] += naccept;
   }
 }
@@ -935,13 +1280,14 @@ size_t metropolis_smem(int N, int k) {
   const int NP = ((N + 31) / 32) * 32;
   return static_cast<size_t>(NP) * (sizeof(double) + sizeof(float)) + 2ull * k * NP * sizeof(T) +
          static_cast<size_t>(NP) * (sizeof(T) + sizeof(float) + sizeof(int)) +
-         static_cast<size_t>(kWin) * (NP + 1) * sizeof(T);
+         static_cast<size_t>(kWin) * (NP + 1) * sizeof(T) +
+         (std::is_same<T, float>::value ? static_cast<size_t>(kRing) * NP * sizeof(T) : 0);
 }
 
 template <typename T>
 cudaError_t launch_metropolis(T* G, int8_t* field, int C, const MetroArgs& a, cudaStream_t st) {
   const int NP = ((a.N + 31) / 32) * 32;
-  const int threads = NP * metro_halves<T>();
+  const int threads = NP * kHalves + (kScalarWarp<T>() ? 32 : 0);
   const size_t sm = metropolis_smem<T>(a.N, a.k);
   cudaError_t e = cudaFuncSetAttribute(k_metropolis<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(sm));
