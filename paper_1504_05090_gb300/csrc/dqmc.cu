@@ -1134,8 +1134,9 @@ int measure_gtau_group(dqmc_ctx* ctx, Group& g, double* dst) {
                     cudaGetLastError()));
     GtauArgs ga{};
     ga.N = g.N; ga.Lx = g.p.Lx; ga.Ly = g.p.Ly; ga.L = g.L;
-    // float-pair groups propagate in their working precision (small tiles,
-    // latency-bound like the wrap); FP64 and FP32 groups in FP64
+    // off the tensor cores, float-pair groups propagate in their working
+    // precision (small tiles, latency-bound like the wrap); FP64 and FP32
+    // groups in FP64
     const bool pair = g.p.precision == DQMC_DF32;
     ga.nv = pair ? (g.tile_wrap > 0 ? std::min(2 * g.tile_wrap, g.N) : std::min(8, g.N))
                  : kron_nv(g, true);
@@ -1148,10 +1149,12 @@ int measure_gtau_group(dqmc_ctx* ctx, Group& g, double* dst) {
     ga.cp = g.d_cp_gtau;
     ga.mat_stride = g.nn();
     ga.bins = g.bins;
-    // FP64 groups on the tensor cores where the tensor-core products are in
-    // use (measured faster than the FP64 pipe); float-pair groups keep their
-    // float-pair propagation, which measured faster than the tensor path
-    const bool tc = ctx->gemm_mode == DQMC_GEMM_TENSOR && g.oz && !pair;
+    // On the tensor cores where the tensor-core products are in use; float-pair
+    // groups only for the larger sides.  The tensor kernel pads both sides to
+    // 16, the float-pair one works for Lx + Ly: 16 x 16, 64 chains, 17 points
+    // 17.2 against 25.7 ms, 8 x 8, 768 chains 12.2 against 11.6 ms; by the work
+    // of both per element they meet near 13 x 13.
+    const bool tc = ctx->gemm_mode == DQMC_GEMM_TENSOR && g.oz && (!pair || g.p.Lx + g.p.Ly >= 28);
     ga.kind = kB; ga.vec_is_col = 1; ga.bin_slot = 0;
     DQ_CLASS(ctx, kTGtauProp);
     DQ_LAUNCH(ctx, tc ? launch_gtau_tc(g.A1, batch, ga, ctx->d_status, g.st)

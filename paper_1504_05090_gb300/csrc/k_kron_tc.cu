@@ -8,17 +8,27 @@
 // memory for all the slices of a call.  Per slice:
 //   x step: rows (vector, y) of length Lx times E_x^T      (M = 128, N = K = 16)
 //   y step: rows (vector, x) of length Ly times E_y^T      (M = 128, N = K = 16)
-// each one digit-sliced product as in k_ozaki.cu: every row of the left
-// operand and every column of the taps is aligned to its largest exponent
-// and cut into eight signed 7-bit digits (exact in BF16), the 36 digit
-// products with p + q <= 7 accumulate in eight FP32 TMEM accumulators, and
-// the epilogue recombines them exactly in 64-bit integers.  Rows and
-// columns past Lx, Ly are zero padding.  The diagonal factor e^{+-c s_l} is
-// an FP64 product per element, before (B, B^{-T}) or after (B^T) the taps.
+// each one digit-sliced product in integer arithmetic: every row of the left
+// operand and the taps are aligned to their largest exponent (55 bits) and cut
+// into seven signed 8-bit digits, -128 .. 127, exact in BF16; the 28 digit
+// products with p + q <= 6 accumulate in seven FP32 TMEM accumulators (sums of
+// 16 products of two digits: exact), and the epilogue puts them together in one
+// 64-bit integer and rounds that to FP64.  What is left out, the products with
+// p + q = 7 of balanced digits, is below that of eight unsigned 7-bit digits
+// with p + q = 8, which need 36 products.  Rows and columns past Lx, Ly are
+// zero padding.  The diagonal factor e^{+-c s_l} is an FP64 product per
+// element, taken with the load of the x step (B, B^{-T}) or the store of the y
+// step (B^T).
 //
-// FP64 work per element and slice: the diagonal product and two
-// recombinations (conversions and one FMA each), against Lx + Ly FMAs for the
-// FP64 Kronecker kernel.
+// What bounds it: the integer and FP32 instructions of the split and the
+// recombination (about 80 per element and step).  The FP64 pipe, which issues a
+// warp instruction in 64 to 76 clocks, is left to the diagonal factor: digits,
+// sums and the rounding use integer and FP32 instructions only, no conversion
+// instruction (15 lanes per clock and SM) among them.  The vectors lie in
+// shared memory with rows of odd length, so that lanes along y and along x both
+// find different banks.  One launch of the 16 x 16 sweep (64 chains x 256
+// vectors x 10 slices): 1.32 ms with eight 7-bit digits, FP64 conversions and
+// rows of Lx, 0.61 ms now.
 #include <cuda_bf16.h>
 
 #include "common.cuh"
@@ -27,7 +37,7 @@
 namespace dqmc {
 namespace {
 
-constexpr int kS = 8;       // digit slices
+constexpr int kS = 7;       // digit slices
 constexpr int kR = 128;     // rows of one product (TMEM lanes)
 constexpr int kK = 16;      // inner dimension (padded side)
 constexpr int kTC = 128;    // threads
@@ -63,64 +73,91 @@ __device__ __forceinline__ bool tc_wait(uint64_t* bar, int parity) {
   return done != 0;
 }
 
-// The 8 digits of x aligned to emax (as k_ozaki.cu), BF16 bit patterns.
-__device__ __forceinline__ void tc_digits(double x, int emax, uint16_t (&dg)[kS]) {
+// Exponent to align a vector to: the largest biased exponent, one higher where
+// the leading seven bits of the significand are all ones, so that the top
+// digit of the aligned number, rounded up by the digits below it, stays below
+// 128.
+__device__ __forceinline__ int tc_exp(double x) {
+  return ((__double2hiint(x) & 0x7FFFFFFF) + 0x4000) >> 20;
+}
+
+// x as the integer round-down(|x| 2^(1077 - emax)) with x's sign, below 2^55,
+// plus 128 in each of its seven bytes: byte 6 - p is then digit p plus 128.
+__device__ __forceinline__ unsigned long long tc_align(double x, int emax) {
   const long long bits = __double_as_longlong(x);
   const int E = static_cast<int>((bits >> 52) & 0x7FF);
-  unsigned long long al = 0ULL;
-  if (E != 0) {
+  long long m = 0;
+  if (E != 0) {  // zero and subnormal inputs contribute zero digits
     const unsigned long long mant =
-        (static_cast<unsigned long long>(bits) & ((1ULL << 52) - 1)) | (1ULL << 52);
-    const int sh = emax - (E - 1023);
-    al = (sh < 64) ? (mant >> sh) : 0ULL;
+        ((static_cast<unsigned long long>(bits) & ((1ULL << 52) - 1)) | (1ULL << 52)) << 2;
+    const int sh = emax - E;
+    m = (sh < 64) ? static_cast<long long>(mant >> sh) : 0LL;
+    if (bits < 0) m = -m;
   }
-  const float sg = (bits < 0) ? -1.0f : 1.0f;
-#pragma unroll
-  for (int p = 0; p < kS; ++p) {
-    const int d = (p < 7) ? static_cast<int>((al >> (46 - 7 * p)) & 127ULL)
-                          : static_cast<int>((al & 15ULL) << 3);
-    const __nv_bfloat16 hb = __float2bfloat16_rn(sg * static_cast<float>(d));
-    dg[p] = *reinterpret_cast<const uint16_t*>(&hb);
-  }
+  return static_cast<unsigned long long>(m) + 0x0080808080808080ULL;
+}
+
+// Digit p of an aligned number as a float: the byte in the low bits of 2^23,
+// minus 2^23 + 128.
+__device__ __forceinline__ float tc_digit(unsigned long long t, int p) {
+  const uint32_t w = (p < 3) ? static_cast<uint32_t>(t >> 32) : static_cast<uint32_t>(t);
+  const int byte = (p < 3) ? 2 - p : 6 - p;
+  return __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7440u | byte)) - 8388736.0f;
+}
+
+// Two floats with at most eight significant bits as a BF16 pair: their high
+// halves.
+__device__ __forceinline__ uint32_t tc_pack(float a, float b) {
+  return __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
 }
 
 // Digits of the taps as the right operand: column j, inner index k,
-// t[(j - k) mod n] for j, k < n (zero padding beyond); column exponents out.
-__device__ void tc_tap_digits(const double* t, int n, unsigned char* bs, int* ex) {
-  for (int j = threadIdx.x; j < kK; j += blockDim.x) {
-    int emax = -100000;
-    for (int k = 0; k < n && j < n; ++k) {
-      const double v = t[((j - k) % n + n) % n];
-      const int E = static_cast<int>((__double_as_longlong(v) >> 52) & 0x7FF);
-      if (E != 0) emax = max(emax, E - 1023);
-    }
-    ex[j] = emax - 6;
-    for (int k = 0; k < kK; ++k) {
-      const double v = (j < n && k < n) ? t[((j - k) % n + n) % n] : 0.0;
-      uint16_t dg[kS];
-      tc_digits(v, emax, dg);
-      for (int p = 0; p < kS; ++p)
-        reinterpret_cast<uint16_t*>(bs + p * kBSlice)[tc_off(j, k)] = dg[p];
-    }
+// t[(j - k) mod n] for j, k < n (zero padding beyond); the columns hold the same
+// taps, so they share one exponent, which is returned.
+__device__ int tc_tap_digits(const double* t, int n, unsigned char* bs) {
+  int emax = 0;
+  for (int k = 0; k < n; ++k) emax = max(emax, tc_exp(t[k]));
+  for (int e = threadIdx.x; e < kK * kK; e += blockDim.x) {
+    const int j = e / kK, k = e - j * kK;
+    const unsigned long long v = tc_align((j < n && k < n) ? t[(j - k + n) % n] : 0.0, emax);
+    for (int p = 0; p < kS; ++p)
+      reinterpret_cast<uint16_t*>(bs + p * kBSlice)[tc_off(j, k)] =
+          static_cast<uint16_t>(__float_as_uint(tc_digit(v, p)) >> 16);
   }
+  return emax;
 }
 
 // Shared-memory state of one CTA of the tensor-core Kronecker kernels.
 struct TcState {
-  unsigned char* as;  // digit slices of the rows (8 x 4 KB)
-  unsigned char* bx;  // digit slices of the taps along x (8 x 512 B)
+  unsigned char* as;  // digit slices of the rows (7 x 4 KB)
+  unsigned char* bx;  // digit slices of the taps along x (7 x 512 B)
   unsigned char* by;  // along y
-  double* V;          // the CTA's vectors [nvpc][N]
+  double* V;          // the CTA's vectors, element (vi, x, y) at vi VP + y LP + x
+  double* sc;         // diagonal of the slice, (x, y) at y LP + x
   uint64_t* mbar;     // MMA completion
-  int* exx;           // column exponents of the taps
-  int* exy;
   int* fail;          // a bounded wait gave up
-  uint32_t tbase;     // TMEM accumulators (8 x 16 columns)
+  int ex, ey;         // exponents of the taps
+  int Lx, Ly, LP, VP;
+  uint32_t tbase;     // TMEM accumulators (7 x 16 columns)
 };
+
+__host__ __device__ __forceinline__ int tc_pitch(int Lx) { return Lx | 1; }
+
+__device__ __forceinline__ void tc_layout(TcState& s, unsigned char* sm, int nvpc, int Lx, int Ly) {
+  s.as = sm;
+  s.bx = s.as + kS * kASlice;
+  s.by = s.bx + kS * kBSlice;
+  s.Lx = Lx;
+  s.Ly = Ly;
+  s.LP = tc_pitch(Lx);
+  s.VP = Ly * s.LP;
+  s.V = reinterpret_cast<double*>(s.by + kS * kBSlice);
+  s.sc = s.V + nvpc * s.VP;
+}
 
 // TMEM, barrier and the digits of the taps of E_x, E_y (kind: E or E^{-1}).
 __device__ void tc_setup(TcState& s, uint32_t* tmem_sh, const KronTaps& taps, bool inv, double* tx,
-                         double* ty, int Lx, int Ly) {
+                         double* ty) {
   const int warp = threadIdx.x >> 5;
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 128;" ::"r"(
@@ -136,9 +173,12 @@ __device__ void tc_setup(TcState& s, uint32_t* tmem_sh, const KronTaps& taps, bo
     tx[threadIdx.x] = inv ? taps.exi[threadIdx.x] : taps.ex[threadIdx.x];
     ty[threadIdx.x] = inv ? taps.eyi[threadIdx.x] : taps.ey[threadIdx.x];
   }
+  // zero digits of k = 8 .. 15, which sides of at most 8 never write
+  for (int e = threadIdx.x; e < kS * kASlice / 16; e += blockDim.x)
+    reinterpret_cast<uint4*>(s.as)[e] = make_uint4(0u, 0u, 0u, 0u);
   __syncthreads();
-  tc_tap_digits(tx, Lx, s.bx, s.exx);
-  tc_tap_digits(ty, Ly, s.by, s.exy);
+  s.ex = tc_tap_digits(tx, s.Lx, s.bx);
+  s.ey = tc_tap_digits(ty, s.Ly, s.by);
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
@@ -153,42 +193,63 @@ __device__ void tc_teardown(const TcState& s) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 128;" ::"r"(s.tbase));
 }
 
-// One factor B on the nv vectors in s.V: the diagonal sc before the taps
+// The number W 2^(e - 2102), W the integer sum of the accumulators, rounded to
+// FP64 (W's leading 53 bits; e: the sum of the two biased exponents).
+__device__ __forceinline__ double tc_compose(long long W, int e) {
+  const unsigned long long x = static_cast<unsigned long long>(W < 0 ? -W : W);
+  const int lz = __clzll(static_cast<long long>(x));
+  const unsigned long long m = ((x << (lz - 1)) + 0x200u) >> 10;  // 2^52 .. 2^53
+  const int ef = e - 1016 - lz;
+  if (x != 0 && (ef < 1 || ef > 2045)) return ldexp(static_cast<double>(W), e - 2102);
+  unsigned long long r = (static_cast<unsigned long long>(ef - 1) << 52) + m;
+  if (W < 0) r |= 0x8000000000000000ULL;
+  return (x == 0) ? 0.0 : __longlong_as_double(static_cast<long long>(r));
+}
+
+// One factor B on the nv vectors in s.V: the diagonal s.sc before the taps
 // (post = false: B, B^{-T}) or after them (post = true: B^T), then the x and
-// y steps as digit-sliced products.  All threads; false if a wait gave up.
-__device__ bool tc_slice(TcState& s, const double* sc, bool post, int nv, int N, int Lx, int Ly,
-                         int& phase) {
+// y steps as digit-sliced products.  All threads, which have synchronised since
+// s.V and s.sc were written; false if a wait gave up.
+__device__ bool tc_slice(TcState& s, bool post, int nv, int& phase) {
   const int warp = threadIdx.x >> 5;
   const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((kK >> 3) << 17) | ((kR >> 4) << 24);
-  double* V = s.V;
-  if (!post)
-    for (int e = threadIdx.x; e < nv * N; e += blockDim.x) V[e] *= sc[e % N];
-  __syncthreads();
   const int r = threadIdx.x;  // the row of both products this thread owns
+  const bool wide = max(s.Lx, s.Ly) > 8;
   for (int dir = 0; dir < 2; ++dir) {
     // row r: (vector, y) with elements x' (x step) or (vector, x) with y' (y step)
-    const int side = dir == 0 ? Ly : Lx, klen = dir == 0 ? Lx : Ly;
+    const int side = dir == 0 ? s.Ly : s.Lx, klen = dir == 0 ? s.Lx : s.Ly;
     const int vi = r / side, o = r - vi * side;
     const bool live = vi < nv;
-    double row[kK];
+    const int base = dir == 0 ? o * s.LP : o, step = dir == 0 ? 1 : s.LP;
+    double* v = s.V + vi * s.VP + base;
+    const double* scp = s.sc + base;
+    int emax = 0;
+    {
+      double row[kK];
 #pragma unroll
-    for (int k = 0; k < kK; ++k) {
-      double v = 0.0;
-      if (live && k < klen) v = (dir == 0) ? V[vi * N + k + Lx * o] : V[vi * N + o + Lx * k];
-      row[k] = v;
-    }
-    int emax = -100000;
+      for (int k = 0; k < kK; ++k) {
+        double x = 0.0;
+        if (live && k < klen) {
+          x = v[k * step];
+          if (!post && dir == 0) x *= scp[k];
+        }
+        row[k] = x;
+        emax = max(emax, tc_exp(x));
+      }
 #pragma unroll
-    for (int k = 0; k < kK; ++k) {
-      const int E = static_cast<int>((__double_as_longlong(row[k]) >> 52) & 0x7FF);
-      if (E != 0) emax = max(emax, E - 1023);
-    }
+      for (int half = 0; half < 2; ++half) {
+        if (half == 1 && !wide) break;
+        unsigned long long t[8];
 #pragma unroll
-    for (int k = 0; k < kK; ++k) {
-      uint16_t dg[kS];
-      tc_digits(row[k], emax, dg);
+        for (int q = 0; q < 8; ++q) t[q] = tc_align(row[half * 8 + q], emax);
 #pragma unroll
-      for (int p = 0; p < kS; ++p) reinterpret_cast<uint16_t*>(s.as + p * kASlice)[tc_off(r, k)] = dg[p];
+        for (int p = 0; p < kS; ++p)
+          *reinterpret_cast<uint4*>(s.as + p * kASlice + 2 * tc_off(r, half * 8)) =
+              make_uint4(tc_pack(tc_digit(t[0], p), tc_digit(t[1], p)),
+                         tc_pack(tc_digit(t[2], p), tc_digit(t[3], p)),
+                         tc_pack(tc_digit(t[4], p), tc_digit(t[5], p)),
+                         tc_pack(tc_digit(t[6], p), tc_digit(t[7], p)));
+      }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;");
@@ -215,12 +276,13 @@ __device__ bool tc_slice(TcState& s, const double* sc, bool post, int nv, int N,
     const bool ok = __syncthreads_and(*s.fail == 0) != 0;
     asm volatile("tcgen05.fence::after_thread_sync;");
     if (!ok) return false;
-    // recombination: (hi + 2^-28 lo) 2^{e_r + f_j - 21}, the power of two in
-    // the exponent field (FP64 products where it would leave the normal
-    // range); the accumulators are read eight columns at a time
-    const int* exj = dir == 0 ? s.exx : s.exy;
+    // recombination, eight columns at a time: the accumulators are integers
+    // below 2^21, read off the low bits of 1.5 2^23 + P_d (as P_d + kM), and
+    // W = sum_d P_d 2^(44 - 8 d) (d = 6 rounded), below 2^63
+    const int e2 = emax + (dir == 0 ? s.ex : s.ey);
 #pragma unroll
     for (int half = 0; half < 2; ++half) {
+      if (half * 8 >= klen) break;
       uint32_t acc[kS][8];
 #pragma unroll
       for (int d = 0; d < kS; ++d) {
@@ -237,36 +299,26 @@ __device__ bool tc_slice(TcState& s, const double* sc, bool post, int nv, int N,
         for (int jq = 0; jq < 8; ++jq) {
           const int j = half * 8 + jq;
           if (j >= klen) continue;
-          long long hi = 0, lo = 0;
+          constexpr uint32_t kM = 0x4B400000u;
+          uint32_t u[kS];
 #pragma unroll
-          for (int d = 0; d < 4; ++d)
-            hi += static_cast<long long>(__float2int_rn(__uint_as_float(acc[d][jq]))) << (7 * (3 - d));
-#pragma unroll
-          for (int d = 4; d < kS; ++d)
-            lo += static_cast<long long>(__float2int_rn(__uint_as_float(acc[d][jq]))) << (7 * (7 - d));
-          const double sum = fma(static_cast<double>(lo), 0x1p-28, static_cast<double>(hi));
-          const int e2 = (emax - 6) + exj[j] - 21;
-          const long long bits = __double_as_longlong(sum);
-          const int E = static_cast<int>((bits >> 52) & 0x7FF), E2 = E + e2;
-          double val;
-          if (E != 0 && E != 0x7FF && E2 > 0 && E2 < 2047)
-            val = __longlong_as_double((bits & ~(0x7FFLL << 52)) | (static_cast<long long>(E2) << 52));
-          else
-            val = sum * ldexp(1.0, emax - 6) * ldexp(1.0, exj[j] - 21);
+          for (int d = 0; d < kS; ++d) u[d] = __float_as_uint(__uint_as_float(acc[d][jq]) + 12582912.0f);
+          const int a = static_cast<int>(u[0] * 256u + u[1] - kM * 257u);
+          const int b = static_cast<int>(u[2] * 256u + u[3] - kM * 257u);
+          const int c = static_cast<int>(u[4] * 256u + u[5] - kM * 257u);
+          const int g = static_cast<int>(u[6] - kM);
+          const long long W = ((static_cast<long long>(a) * 65536 + b) << 20) +
+                              (static_cast<long long>(c) << 4) + ((g + 8) >> 4);
+          double val = tc_compose(W, e2);
           // rows are read above and written only here, each by its owner
-          if (dir == 0)
-            V[vi * N + j + Lx * o] = val;
-          else
-            V[vi * N + o + Lx * j] = val;
+          if (post && dir == 1) val *= scp[j * step];
+          v[j * step] = val;
         }
       }
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
   }
-  if (post)
-    for (int e = threadIdx.x; e < nv * N; e += blockDim.x) V[e] *= sc[e % N];
-  __syncthreads();
   return true;
 }
 
@@ -294,43 +346,39 @@ __global__ void __launch_bounds__(kTC) k_kron_tc(const double* in, double* out, 
   extern __shared__ __align__(1024) unsigned char tc_sm[];
   __shared__ uint64_t mbar;
   __shared__ uint32_t tmem_sh;
-  __shared__ int exx[kK], exy[kK], fail_sh;
-  __shared__ double tx[kMaxSide], ty[kMaxSide], sc[kMaxN];
+  __shared__ int fail_sh;
+  __shared__ double tx[kMaxSide], ty[kMaxSide];
   TcState s;
-  s.as = tc_sm;
-  s.bx = s.as + kS * kASlice;
-  s.by = s.bx + kS * kBSlice;
-  s.V = reinterpret_cast<double*>(s.by + kS * kBSlice);
+  tc_layout(s, tc_sm, nvpc, a.Lx, a.Ly);
   s.mbar = &mbar;
-  s.exx = exx;
-  s.exy = exy;
   s.fail = &fail_sh;
   const double* src = in + static_cast<size_t>(b) * a.mat_stride;
-  for (int e = threadIdx.x; e < nvpc * N; e += blockDim.x) {
-    const int vi = e / N, i = e - vi * N;
-    double val = 0.0;
-    if (vi < nv) {
-      val = src[static_cast<size_t>(v0 + vi) * N + i];
-      if (a.vscale) val *= a.vscale[static_cast<size_t>(b) * a.vscale_stride + v0 + vi];
-    }
-    s.V[e] = val;
+  for (int e = threadIdx.x; e < nv * N; e += blockDim.x) {
+    const int vi = e / N, i = e - vi * N, y = i / a.Lx;
+    double val = src[static_cast<size_t>(v0) * N + e];
+    if (a.vscale) val *= a.vscale[static_cast<size_t>(b) * a.vscale_stride + v0 + vi];
+    s.V[vi * s.VP + y * s.LP + i - y * a.Lx] = val;
   }
-  tc_setup(s, &tmem_sh, a.taps, a.kind == kBIT, tx, ty, a.Lx, a.Ly);
+  tc_setup(s, &tmem_sh, a.taps, a.kind == kBIT, tx, ty);
   const double up = (a.kind == kBIT) ? a.emc : a.ec, dn = (a.kind == kBIT) ? a.ec : a.emc;
   const int8_t* f = a.field + static_cast<size_t>(chain) * a.L * N;
   int phase = 0;
   bool ok = true;
   for (int stp = 0; stp < count && ok; ++stp) {
     const int l0 = first + stp * a.dir;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) sc[i] = f[static_cast<size_t>(l0) * N + i] > 0 ? up : dn;
+    for (int i = threadIdx.x; i < N; i += blockDim.x) {
+      const int y = i / a.Lx;
+      s.sc[y * s.LP + i - y * a.Lx] = f[static_cast<size_t>(l0) * N + i] > 0 ? up : dn;
+    }
     __syncthreads();
-    ok = tc_slice(s, sc, a.kind == kBT, nv, N, a.Lx, a.Ly, phase);
+    ok = tc_slice(s, a.kind == kBT, nv, phase);
   }
   if (!ok && threadIdx.x == 0) atomicExch(status, kDevTimeout);
+  __syncthreads();
   double* dst = out + static_cast<size_t>(b) * a.out_stride;
   for (int e = threadIdx.x; e < nv * N; e += blockDim.x) {
-    const int vi = e / N, i = e - vi * N;
-    dst[static_cast<size_t>(v0 + vi) * N + i] = s.V[e];
+    const int vi = e / N, i = e - vi * N, y = i / a.Lx;
+    dst[static_cast<size_t>(v0) * N + e] = s.V[vi * s.VP + y * s.LP + i - y * a.Lx];
   }
   tc_teardown(s);
 }
@@ -339,7 +387,8 @@ __global__ void __launch_bounds__(kTC) k_kron_tc(const double* in, double* out, 
 // of one stabilisation point's G(c,0)^T (kind B) or Y (kind B^{-T}) are
 // propagated over the slices of its block, and after each slice every
 // element is added to the bin of its separation (spin-up G(l,0) bins or Y
-// bins of slice l), first in shared memory, then into bins[chain][l][slot].
+// bins of slice l): one thread per bin sums its element of each of the CTA's
+// vectors and adds the sum to bins[chain][l][slot].
 __global__ void __launch_bounds__(kTC) k_gtau_tc(const double* Xall, GtauArgs a, int nvpc,
                                                 int* status) {
   const int b = blockIdx.y;
@@ -351,48 +400,51 @@ __global__ void __launch_bounds__(kTC) k_gtau_tc(const double* Xall, GtauArgs a,
   extern __shared__ __align__(1024) unsigned char tc_sm[];
   __shared__ uint64_t mbar;
   __shared__ uint32_t tmem_sh;
-  __shared__ int exx[kK], exy[kK], fail_sh;
-  __shared__ double tx[kMaxSide], ty[kMaxSide], sc[kMaxN], sbin[kMaxN];
+  __shared__ int fail_sh;
+  __shared__ double tx[kMaxSide], ty[kMaxSide];
   TcState s;
-  s.as = tc_sm;
-  s.bx = s.as + kS * kASlice;
-  s.by = s.bx + kS * kBSlice;
-  s.V = reinterpret_cast<double*>(s.by + kS * kBSlice);
+  tc_layout(s, tc_sm, nvpc, a.Lx, a.Ly);
   s.mbar = &mbar;
-  s.exx = exx;
-  s.exy = exy;
   s.fail = &fail_sh;
   const double* X = Xall + static_cast<size_t>(b) * a.mat_stride;
-  for (int e = threadIdx.x; e < nvpc * N; e += blockDim.x) {
-    const int vi = e / N, i = e - vi * N;
-    s.V[e] = (vi < nv) ? X[static_cast<size_t>(v0 + vi) * N + i] : 0.0;
+  for (int e = threadIdx.x; e < nv * N; e += blockDim.x) {
+    const int vi = e / N, i = e - vi * N, y = i / a.Lx;
+    s.V[vi * s.VP + y * s.LP + i - y * a.Lx] = X[static_cast<size_t>(v0) * N + e];
   }
-  for (int i = threadIdx.x; i < N; i += blockDim.x) sbin[i] = 0.0;
-  tc_setup(s, &tmem_sh, a.taps, a.kind == kBIT, tx, ty, a.Lx, a.Ly);
-  const Geom g{a.Lx, a.Ly, N};
+  tc_setup(s, &tmem_sh, a.taps, a.kind == kBIT, tx, ty);
   const int8_t* f = a.field + static_cast<size_t>(chain) * a.L * N;
   const double up = (a.kind == kBIT) ? a.emc : a.ec, dn = (a.kind == kBIT) ? a.ec : a.emc;
   int phase = 0;
   bool ok = true;
   for (int l = lo; l < hi && ok; ++l) {
     if (l > lo) {
-      for (int i = threadIdx.x; i < N; i += blockDim.x)
-        sc[i] = f[static_cast<size_t>(l - 1) * N + i] > 0 ? up : dn;
+      for (int i = threadIdx.x; i < N; i += blockDim.x) {
+        const int y = i / a.Lx;
+        s.sc[y * s.LP + i - y * a.Lx] = f[static_cast<size_t>(l - 1) * N + i] > 0 ? up : dn;
+      }
       __syncthreads();
-      ok = tc_slice(s, sc, false, nv, N, a.Lx, a.Ly, phase);
+      ok = tc_slice(s, false, nv, phase);
       if (!ok) break;
     }
-    for (int e = threadIdx.x; e < nv * N; e += blockDim.x) {
-      const int vi = e / N, el = e - vi * N;
-      const int q = v0 + vi;
-      const int sep = a.vec_is_col ? sep_index(el, q, g) : sep_index(q, el, g);
-      atomicAdd(&sbin[sep], s.V[e]);
-    }
-    __syncthreads();
     double* out = a.bins + ((static_cast<size_t>(chain) * (a.L + 1) + l) * 2 + a.bin_slot) * N;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
-      atomicAdd(&out[i], sbin[i]);
-      sbin[i] = 0.0;
+    for (int r = threadIdx.x; r < N; r += blockDim.x) {
+      const int ry = r / a.Lx, rx = r - ry * a.Lx;
+      int qy = v0 / a.Lx, qx = v0 - qy * a.Lx;
+      double sum = 0.0;
+      for (int vi = 0; vi < nv; ++vi) {
+        // vec_is_col: r = r_el - r_q, else r = r_q - r_el
+        int x = a.vec_is_col ? qx + rx : qx - rx, y = a.vec_is_col ? qy + ry : qy - ry;
+        if (x < 0) x += a.Lx;
+        if (x >= a.Lx) x -= a.Lx;
+        if (y < 0) y += a.Ly;
+        if (y >= a.Ly) y -= a.Ly;
+        sum += s.V[vi * s.VP + y * s.LP + x];
+        if (++qx == a.Lx) {
+          qx = 0;
+          ++qy;
+        }
+      }
+      atomicAdd(&out[r], sum);
     }
     __syncthreads();
   }
@@ -402,16 +454,16 @@ __global__ void __launch_bounds__(kTC) k_gtau_tc(const double* Xall, GtauArgs a,
 
 int kron_tc_vectors(int Lx, int Ly) { return kR / max(Lx, Ly); }
 
-static size_t tc_bytes(int nvpc, int N) {
+static size_t tc_bytes(int nvpc, int Lx, int Ly) {
   return static_cast<size_t>(kS) * kASlice + 2ull * kS * kBSlice +
-         static_cast<size_t>(nvpc) * N * sizeof(double);
+         static_cast<size_t>(nvpc + 1) * Ly * tc_pitch(Lx) * sizeof(double);
 }
 
 cudaError_t launch_kron_tc(const double* in, double* out, int batch, const KronArgs& a, int* status,
                            cudaStream_t st) {
   if (a.Lx > kK || a.Ly > kK) return cudaErrorInvalidValue;
   const int nvpc = kron_tc_vectors(a.Lx, a.Ly);
-  const size_t smem = tc_bytes(nvpc, a.N);
+  const size_t smem = tc_bytes(nvpc, a.Lx, a.Ly);
   cudaError_t e = cudaFuncSetAttribute(k_kron_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem));
   if (e != cudaSuccess) return e;
@@ -424,7 +476,7 @@ cudaError_t launch_gtau_tc(const double* X, int batch, const GtauArgs& a, int* s
                            cudaStream_t st) {
   if (a.Lx > kK || a.Ly > kK) return cudaErrorInvalidValue;
   const int nvpc = kron_tc_vectors(a.Lx, a.Ly);
-  const size_t smem = tc_bytes(nvpc, a.N);
+  const size_t smem = tc_bytes(nvpc, a.Lx, a.Ly);
   cudaError_t e = cudaFuncSetAttribute(k_gtau_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem));
   if (e != cudaSuccess) return e;
