@@ -16,7 +16,7 @@
 //
 //   for each panel of w <= kNB columns (rows c0 .. n - 1):
 //     k_qrb_panel  sort the remaining columns, FP64 Householder QR of the
-//                  panel in shared memory with local pivoting, the compact-WY
+//                  panel in registers with local pivoting, the compact-WY
 //                  factor T of its reflectors (H_0 ... H_{w-1} = I - V T V^T)
 //                  and Y = T^T V^T;
 //     trailing columns A <- (I - V T^T V^T) A = A - V (Y A), written in the
@@ -43,6 +43,7 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "qr_scalars.cuh"
 
 namespace dqmc {
 namespace {
@@ -50,11 +51,6 @@ namespace {
 namespace cg = cooperative_groups;
 
 constexpr int kNB = 32;  // panel width
-
-__device__ __forceinline__ double qb_wsum(double v) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-  return v;
-}
 
 // log2 of the squared norm of x[0 .. len) as an FP32 sort key, from the
 // exponent fields and the FP32 mantissas (the order only steers the
@@ -96,85 +92,86 @@ __device__ __forceinline__ float qb_norm_key(const double* x, int len, int lane)
   return 2.0f * static_cast<float>(emax - 1023) + __log2f(s);
 }
 
-// Warp sums of four values per lane: lanes 8q .. 8q + 7 end with the sum of
-// value q, which is broadcast back to every lane (6 FP64 additions instead
-// of 20: the first two butterfly stages exchange the halves each lane gives
-// away).
-__device__ __forceinline__ void qb_wsum4(double (&a)[4]) {
-  const int lane = threadIdx.x & 31;
-  const bool lo16 = lane < 16;
-  const double s0 = lo16 ? a[2] : a[0], s1 = lo16 ? a[3] : a[1];
-  const double k0 = lo16 ? a[0] : a[2], k1 = lo16 ? a[1] : a[3];
-  const double b0 = k0 + __shfl_xor_sync(0xFFFFFFFFu, s0, 16);
-  const double b1 = k1 + __shfl_xor_sync(0xFFFFFFFFu, s1, 16);
-  const bool hi8 = (lane & 8) != 0;
-  double c = (hi8 ? b1 : b0) + __shfl_xor_sync(0xFFFFFFFFu, hi8 ? b0 : b1, 8);
-  c += __shfl_xor_sync(0xFFFFFFFFu, c, 4);
-  c += __shfl_xor_sync(0xFFFFFFFFu, c, 2);
-  c += __shfl_xor_sync(0xFFFFFFFFu, c, 1);
-#pragma unroll
-  for (int q = 0; q < 4; ++q) a[q] = __shfl_sync(0xFFFFFFFFu, c, 8 * q);
+constexpr int kPCS = 4;             // CTAs per matrix (one cluster)
+constexpr int kPCW = kNB / kPCS;    // column warps per CTA
+constexpr int kPW = 16;             // warps per CTA: columns, scalars, copies
+constexpr int kPT = 32 * kPW;
+
+// x 2^-e on the exponent field; what would leave the range of normal numbers
+// becomes zero.  Inf and NaN stay.
+__device__ __forceinline__ double qb_shift(double x, int e) {
+  const long long b = __double_as_longlong(x);
+  const int ex = static_cast<int>((b >> 52) & 0x7FF), f = ex - e;
+  if (ex == 0x7FF || f >= 0x7FF) return x;
+  if (ex == 0 || f <= 0) return 0.0;
+  return __longlong_as_double(b - (static_cast<long long>(e) << 52));
 }
 
-constexpr int kPT = 512;  // threads of each CTA of the panel kernel
-
-// Rows of a panel per CTA: the pair of CTAs of a matrix splits the m rows,
-// CTA 0 taking rows [0, h) with h >= w, so that the diagonal block (rows
-// q < w, where the reflectors start and R ends) is entirely its own.
-__host__ __device__ __forceinline__ int qb_split(int m, int w) {
-  const int half = (m + 1) / 2;
-  const int h = half > w ? half : w;
-  return h < m ? h : m;
+__device__ __forceinline__ int qb_exp(double x) {  // floor(log2 |x|), 0 for x = 0
+  const int ex = (__double2hiint(x) >> 20) & 0x7FF;
+  return ex ? ex - 1023 : 0;
 }
 
-// One exchange between the two CTAs of a matrix (distributed shared memory):
-// a[r][s] is CTA r's partial sum for panel column s, b[s] a value that only
-// CTA 0 holds (an entry of the diagonal block).
-struct QbXch {
-  double a[2][kNB];
-  double b[kNB];
+// A CTA's best column for a step: sigma, the pivot key (0: no live column) and
+// the column.
+struct QbCand {
+  double sigma;
+  unsigned key;
+  int col;
 };
 
-// One panel, one cluster of two CTAs per matrix, the panel's rows split
-// between them (qb_split); rows of the transposed storage are columns of X;
-// `src` holds the matrix after the previous panel (the input X^T for the
-// first), `dst` receives the rows c0 .. n - 1.
+__device__ __forceinline__ void qb_bar(int id, int threads) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+// One panel, one cluster of four CTAs per matrix; rows of the transposed
+// storage are columns of X; `src` holds the matrix after the previous panel
+// (the input X^T for the first), `dst` receives the rows c0 .. n - 1.
+//
+// What bounds it: the chain of w Householder steps.  The work of a step is
+// small (an FP64 warp instruction takes its SM quarter 64 to 76 clocks, and a
+// step has a few per warp), so the kernel is laid out for a short chain: a
+// warp per panel column, the column in registers (row c0 + lane + 32 t in
+// x[t]), eight columns per CTA; sums over the lanes in integer arithmetic; the
+// scalars of the reflector in one warp beside the dot products, without
+// sqrt() and division; and one cluster barrier per step, which carries each
+// CTA's candidate for the next pivot column with its sigma, prepared before
+// the other columns' norms are touched again.
+//
 //  1. Sort: the rows c >= c0 of src by the norm of their entries c0 .. n - 1
-//     (each CTA finds the keys of half of them and writes them to both);
-//     rank w .. m - 1 go to dst rows c0 + w .. n - 1 (whole rows), perm
-//     follows.
-//  2. The w largest are the panel: P[q][rl] = entry c0 + r0 + rl of panel
-//     column q for the CTA's rows r0 + rl.  Step q (as LAPACK's xGEQP3 within
-//     the panel): take the panel column of largest remaining norm (rows q ..)
-//     into position q, the reflector H_q = I - tau_q v_q v_q^T with v_q[q] = 1
-//     that maps P[q][q..m) to beta_q e_q, applied to the panel columns
-//     q + 1 .. w - 1.  The norms are not downdated: the same pass that
-//     applies H_q sums the squares of every column's rows q + 2 .. (the
-//     reflector's sigma at the next step) and CTA 0 reads off row q + 1, so
-//     that both CTAs hold the exact alpha^2 + sigma of every candidate.
-//     Two exchanges per step, each closed by a cluster barrier (the same
-//     number in both CTAs, independent of the data): the partial dot
-//     products v_q . x_s, then the partial sums of squares with row q + 1.
-//     Every value both CTAs use is summed in the same order on both, so
-//     their pivots and reflector scalars are identical.
-//  3. Gram matrix V^T V from the partial sums of both CTAs; T column by
-//     column, T[0:q, q] = -tau_q T[0:q, 0:q] (V^T v_q)[0:q], T[q][q] = tau_q
-//     (on both CTAs); then Y = T^T V^T for the CTA's rows.
+//     (each CTA finds the keys of a quarter of them and writes them to all).
+//     The w largest are the panel, column i with warp i / 4 of CTA i mod 4.
+//     Ranks w .. m - 1 go to dst rows c0 + w .. n - 1 (whole rows, copied by
+//     spare warps beside step 2), perm follows.
+//  2. Step j (as k_qr_smem): x_p the pivot, s = |x_p[j..)|, v = x_p[j..) with
+//     v[j] = sign(x_p[j]) (|x_p[j]| + s), H = I - kap v v^T.  Every column's
+//     warp forms g = v . x_s: for a column not yet chosen the factor
+//     c = kap g, R_js and the downdated norm (summed afresh as in k_qr_smem),
+//     then x_s -= c v; for a finished column, whose registers hold v_s, the
+//     entry v_s . v_j of the Gram matrix.
+//  3. H_0 ... H_{w-1} = I - V T V^T with T[0:q, q] = -kap_q T[0:q, 0:q] (V^T
+//     v_q)[0:q], T[q][q] = kap_q, a column of T per step by the warp of the
+//     scalars.  V leaves scaled by powers of two to 1 <= |v_q[q]| < 2 (the
+//     digit-sliced products that follow add over q), T with it.  Then
+//     Y = T^T V^T, 32 rows at a time spread over the CTAs.
 //  4. Panel rows to dst rows c0 .. c0 + w - 1 (entries below c0 moved with
-//     their column, R on and above the diagonal, beta_q on it, v_q below),
-//     v_q to row c0 + q of Vt, Y to rows c0 .. of Yt (entries c0 ..),
-//     D[c0 + q] = |beta_q|, perm.
-__global__ void __launch_bounds__(kPT) k_qrb_panel(const double* Wsall, long long sWs, double* Wdall,
-                                                  long long sWd, int* permall, double* Vall,
-                                                  long long sV, double* Yall, long long sY,
-                                                  double* Dall, long long sD, int n, int c0, int w,
-                                                  int* status) {
+//     their column, R on and above the diagonal), v_q to row c0 + q of Vt, Y
+//     to rows c0 .. of Yt (entries c0 ..), D[c0 + q] = |beta_q|, perm.
+//
+// A whole factorisation at n = 256 (with its 30 products, about 1.4 ms of it):
+// 4 matrices 2.98 -> 1.89 ms, 64: 3.49 -> 2.71 ms, 128: 6.51 -> 4.86 ms; n =
+// 160, 16 matrices: 1.69 -> 1.08 ms.  Before: a pair of CTAs with the rows
+// split, columns in shared memory, two exchanges per step and sqrt() and a
+// division in the chain.
+__global__ void __launch_bounds__(kPT, 2) k_qrb_panel(const double* Wsall, long long sWs, double* Wdall,
+                                                     long long sWd, int* permall, double* Vall,
+                                                     long long sV, double* Yall, long long sY,
+                                                     double* Dall, long long sD, int n, int c0, int w,
+                                                     int* status) {
   cg::cluster_group cl = cg::this_cluster();
-  const int rank = static_cast<int>(cl.block_rank()), peer = rank ^ 1;
-  const int b = blockIdx.x >> 1;
-  const int m = n - c0;
-  const int h = qb_split(m, w);
-  const int r0 = rank ? h : 0, ml = (rank ? m : h) - r0;  // this CTA's rows r0 .. r0 + ml - 1
+  const int rank = static_cast<int>(cl.block_rank());
+  const int b = blockIdx.x / kPCS;
+  const int m = n - c0, nt = (m + 31) / 32, mp = 32 * nt;
   const double* Ws = Wsall + b * sWs;
   double* Wd = Wdall + b * sWd;
   int* perm = permall + static_cast<long long>(b) * n;
@@ -182,323 +179,311 @@ __global__ void __launch_bounds__(kPT) k_qrb_panel(const double* Wsall, long lon
   double* Yt = Yall + b * sY;
   double* D = Dall + b * sD;
   extern __shared__ __align__(16) double qb_sm[];
-  double* P = qb_sm;  // [w][ml]
+  double* Vb = qb_sm;            // [w][mp] reflectors
+  double* buf = qb_sm + w * mp;  // [2][kPCS][mp] candidates by step parity and CTA
   __shared__ float key[kMaxN];
-  __shared__ int src_of[kMaxN];  // rank -> source row - c0
-  __shared__ int pold[kMaxN];    // perm[c0 ..] on entry
+  __shared__ short src_of[kMaxN];  // rank -> source row - c0
+  __shared__ int pold[kMaxN];      // perm[c0 ..] on entry
   __shared__ double T[kNB][kNB + 1];
-  __shared__ double Gp[2][kNB][kNB + 1];  // Gram partials of the two CTAs, [s][q] for s < q
-  __shared__ QbXch xch[2];
-  __shared__ double taus[kNB], betas[kNB], sig[kNB], alp[kNB];
-  __shared__ double scal_sh;
-  __shared__ int lp[kNB];  // panel position -> rank of its column
-  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  __shared__ double G[kNB][kNB + 1];  // v_s . v_q, s < q
+  __shared__ double kaps[kNB], betas[kNB], vjs[kNB];
+  __shared__ QbCand cand[2][kPCS];
+  __shared__ unsigned keys[2][kPCW];
+  __shared__ unsigned char wait_sum[kPCW];
+  __shared__ double kap_sh, vj_sh;
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  constexpr int kR = kMaxN / 32;
 
   // 1. sort the remaining columns
-  {
-    float* key_peer = cl.map_shared_rank(key, peer);
-    const int kh = (m + 1) / 2, k0 = rank ? kh : 0, k1 = rank ? m : kh;
-    for (int c = k0 + wp; c < k1; c += nw) {
-      const float k = qb_norm_key(Ws + static_cast<size_t>(c0 + c) * n + c0, m, lane);
-      if (lane == 0) {
-        key[c] = k;
-        key_peer[c] = k;
-      }
-    }
+  cl.sync();  // the peers run: their shared memory may be written
+  for (int c = rank + kPCS * wp; c < m; c += kPCS * kPW) {
+    const float k = qb_norm_key(Ws + static_cast<size_t>(c0 + c) * n + c0, m, lane);
+    if (lane < kPCS) *cl.map_shared_rank(key + c, lane) = k;
   }
-  for (int i = threadIdx.x; i < m; i += blockDim.x) pold[i] = (c0 == 0) ? i : perm[c0 + i];
+  for (int i = threadIdx.x; i < m; i += kPT) pold[i] = (c0 == 0) ? i : perm[c0 + i];
   cl.sync();
-  for (int i = threadIdx.x; i < m; i += blockDim.x) {
+  for (int i = threadIdx.x; i < m; i += kPT) {
     const float ki = key[i];
     int rk = 0;
     for (int i2 = 0; i2 < m; ++i2) {
       const float k2 = key[i2];
       rk += (k2 > ki || (k2 == ki && i2 < i)) ? 1 : 0;
     }
-    src_of[rk] = i;
+    src_of[rk] = static_cast<short>(i);
   }
   __syncthreads();
-  {  // whole rows, a warp per row (rows interleaved between the CTAs), all
-     // loads of a lane in flight before its stores
-    constexpr int kR = kMaxN / 32;
-    for (int pos = w + rank * nw + wp; pos < m; pos += 2 * nw) {
-      const double* srow = Ws + static_cast<size_t>(c0 + src_of[pos]) * n;
-      double* drow = Wd + static_cast<size_t>(c0 + pos) * n;
-      double t[kR];
+
+  // 2. the panel
+  double x[kR];
+  int step = -1;                     // of this warp's column
+  const int cid = rank + kPCS * wp;  // the column (column warps)
+  if (wp < kPCW) {
+    const bool exists = cid < w;
+    bool live = exists;
+    int es = 0;
 #pragma unroll
-      for (int u = 0; u < kR; ++u) t[u] = (lane + 32 * u < n) ? srow[lane + 32 * u] : 0.0;
+    for (int t = 0; t < kR; ++t) {
+      const int r = lane + 32 * t;
+      x[t] = (exists && r < m) ? Ws[static_cast<size_t>(c0 + src_of[cid]) * n + c0 + r] : 0.0;
+    }
+    auto sumsq = [&](int j) {  // rows > j
+      double a = (lane > j) ? x[0] * x[0] : 0.0;
 #pragma unroll
-      for (int u = 0; u < kR; ++u)
-        if (lane + 32 * u < n) drow[lane + 32 * u] = t[u];
-    }
-  }
-  if (rank == 0)
-    for (int pos = w + threadIdx.x; pos < m; pos += blockDim.x) perm[c0 + pos] = pold[src_of[pos]];
-  // 2. the panel: this CTA's rows of the w columns
-  {
-    constexpr int kU = kNB * kMaxN / 2 / kPT;
-    double t[kU];
+      for (int t = 1; t < kR; ++t)
+        if (t < nt) a = fma(x[t], x[t], a);
+      return a;
+    };
+    auto pick = [&](const unsigned* ks) {  // warp of the largest key, -1: none
+      const unsigned k = (lane < kPCW) ? ks[lane] : 0u;
+      const unsigned km = __reduce_max_sync(0xFFFFFFFFu, k);
+      return km ? __ffs(__ballot_sync(0xFFFFFFFFu, k == km)) - 1 : -1;
+    };
+    auto key_of = [](double v) { return (static_cast<unsigned>(__double2hiint(v)) & 0x7FFFFFFFu) + 1u; };
+    // this warp's column as the CTA's candidate for step j (has: false: no
+    // live column left)
+    auto send = [&](int j, bool has, unsigned k) {
+      QbCand cd{0.0, 0u, kNB};
+      if (has) {
 #pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      const int e = threadIdx.x + u * kPT, q = e / max(ml, 1), rl = e - q * max(ml, 1);
-      t[u] = (e < w * ml) ? Ws[static_cast<size_t>(c0 + src_of[q]) * n + c0 + r0 + rl] : 0.0;
-    }
+        for (int t = 0; t < kR; ++t)
+          if (t < nt)
 #pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      const int e = threadIdx.x + u * kPT;
-      if (e < w * ml) P[e] = t[u];
-    }
-  }
-  if (threadIdx.x < w) lp[threadIdx.x] = threadIdx.x;
-  __syncthreads();
-  int xk = 0;  // exchanges so far; exchange k uses slot k & 1
-  {  // sigma (rows 1 ..) and alpha (row 0) of every column before step 0
-    QbXch* mine = &xch[0];
-    QbXch* theirs = cl.map_shared_rank(mine, peer);
-    for (int q = wp; q < w; q += nw) {
-      double a = 0.0;
-      for (int rl = lane; rl < ml; rl += 32)
-        if (r0 + rl > 0) a = fma(P[q * ml + rl], P[q * ml + rl], a);
-      a = qb_wsum(a);
-      if (lane == 0) {
-        mine->a[rank][q] = a;
-        theirs->a[rank][q] = a;
-        if (rank == 0) {
-          mine->b[q] = P[q * ml];
-          theirs->b[q] = P[q * ml];
-        }
+            for (int q = 0; q < kPCS; ++q)
+              *cl.map_shared_rank(buf + ((j & 1) * kPCS + rank) * mp + lane + 32 * t, q) = x[t];
+        cd.sigma = qs_warp_sum_pos(sumsq(j));
+        cd.key = k;
+        cd.col = cid;
       }
-    }
-    cl.sync();
-    if (threadIdx.x < w) {
-      sig[threadIdx.x] = mine->a[0][threadIdx.x] + mine->a[1][threadIdx.x];
-      alp[threadIdx.x] = mine->b[threadIdx.x];
-    }
-    xk = 1;
-    __syncthreads();
-  }
-  constexpr int kRPL = kMaxN / 2 / 32;  // local rows per lane (ml <= 128)
-  for (int q = 0; q < w; ++q) {
-    double* x = P + static_cast<size_t>(q) * ml;
-    if (wp == 0) {
-      // pivot: largest alpha^2 + sigma among positions q .. w - 1 (compared
-      // in FP32: the keys only choose the order)
-      const int s = q + lane;
-      float kv = (s < w) ? static_cast<float>(fma(alp[s], alp[s], sig[s])) : -1.0f;
-      int ks = (s < w) ? s : w;
-      for (int o = 16; o > 0; o >>= 1) {
-        const float kv2 = __shfl_xor_sync(0xFFFFFFFFu, kv, o);
-        const int ks2 = __shfl_xor_sync(0xFFFFFFFFu, ks, o);
-        if (kv2 > kv || (kv2 == kv && ks2 < ks)) {
-          kv = kv2;
-          ks = ks2;
-        }
-      }
-      const int piv = (ks < w) ? ks : q;
-      if (piv != q) {
-        double* y = P + static_cast<size_t>(piv) * ml;
-        for (int rl = lane; rl < ml; rl += 32) {
-          const double t = x[rl];
-          x[rl] = y[rl];
-          y[rl] = t;
-        }
-        if (lane == 0) {
-          double t = sig[q];
-          sig[q] = sig[piv];
-          sig[piv] = t;
-          t = alp[q];
-          alp[q] = alp[piv];
-          alp[piv] = t;
-          const int ti = lp[q];
-          lp[q] = lp[piv];
-          lp[piv] = ti;
-        }
-      }
-      __syncwarp();
-      if (lane == 0) {  // reflector scalars, the same on both CTAs
-        const double alpha = alp[q], sg = sig[q];
-        double tau = 0.0, beta = alpha, scal = 1.0;
-        if (sg != 0.0) {
-          const double nr = sqrt(fma(alpha, alpha, sg));
-          beta = (alpha <= 0.0) ? nr : -nr;
-          // tau = (beta - alpha) / beta and scal = 1 / (alpha - beta) from
-          // one reciprocal
-          const double am = alpha - beta, rb = 1.0 / (beta * am);
-          tau = -(am * am) * rb;
-          scal = beta * rb;
-        }
-        taus[q] = tau;
-        betas[q] = beta;
-        scal_sh = scal;
-      }
-    }
-    __syncthreads();
-    const double tau = taus[q], scal = scal_sh;
-    for (int rl = threadIdx.x; rl < ml; rl += blockDim.x)
-      if (r0 + rl > q) x[rl] *= scal;
-    __syncthreads();
-    // columns s0 .. s0 + 3 per warp (one group: 4 x 16 warps > kNB)
-    const int s0 = q + 1 + 4 * wp;
-    const bool has = s0 < w;
-    double xv[4][kRPL], vr[kRPL];
+      if (lane < kPCS) *cl.map_shared_rank(&cand[j & 1][rank], lane) = cd;
+    };
+    double n1 = qs_warp_sum_pos(sumsq(-1)), n2 = n1;
+    if (lane == 0) keys[0][wp] = live ? key_of(n1) : 0u;
+    qb_bar(2, 32 * kPCW);
     {
-      QbXch* mine = &xch[xk & 1];
-      QbXch* theirs = cl.map_shared_rank(mine, peer);
-      if (has) {
-        double acc[4] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll
-        for (int t = 0; t < kRPL; ++t) {
-          const int rl = lane + 32 * t, r = r0 + rl;
-          vr[t] = (rl < ml && r >= q) ? ((r == q) ? 1.0 : x[rl]) : 0.0;
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            xv[u][t] = (s0 + u < w && rl < ml) ? P[static_cast<size_t>(s0 + u) * ml + rl] : 0.0;
-            acc[u] = fma(vr[t], xv[u][t], acc[u]);
-          }
-        }
-        qb_wsum4(acc);
-        if (lane == 0)
-#pragma unroll
-          for (int u = 0; u < 4; ++u)
-            if (s0 + u < w) {
-              mine->a[rank][s0 + u] = acc[u];
-              theirs->a[rank][s0 + u] = acc[u];
-            }
-      }
-      cl.sync();
-      ++xk;
-      QbXch* mine2 = &xch[xk & 1];
-      QbXch* theirs2 = cl.map_shared_rank(mine2, peer);
-      if (has) {
-        // apply H_q; sums of squares of rows q + 2 .., row q + 1 read off
-        double sq[4] = {0.0, 0.0, 0.0, 0.0}, nx[4] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int su = (s0 + u < w) ? s0 + u : s0;
-          const double dt = tau * (mine->a[0][su] + mine->a[1][su]);
-#pragma unroll
-          for (int t = 0; t < kRPL; ++t) {
-            const int rl = lane + 32 * t, r = r0 + rl;
-            if (s0 + u < w && rl < ml) {
-              if (r >= q) {
-                xv[u][t] = fma(-dt, vr[t], xv[u][t]);
-                P[static_cast<size_t>(s0 + u) * ml + rl] = xv[u][t];
-              }
-              if (r > q + 1) sq[u] = fma(xv[u][t], xv[u][t], sq[u]);
-              if (r == q + 1) nx[u] = xv[u][t];
-            }
-          }
-        }
-        qb_wsum4(sq);
-        // row q + 1 < w is on CTA 0, lane q + 1 (t = 0): broadcast it
-#pragma unroll
-        for (int u = 0; u < 4; ++u) nx[u] = __shfl_sync(0xFFFFFFFFu, nx[u], (q + 1) & 31);
-        if (lane == 0)
-#pragma unroll
-          for (int u = 0; u < 4; ++u)
-            if (s0 + u < w) {
-              mine2->a[rank][s0 + u] = sq[u];
-              theirs2->a[rank][s0 + u] = sq[u];
-              if (rank == 0) {
-                mine2->b[s0 + u] = nx[u];
-                theirs2->b[s0 + u] = nx[u];
-              }
-            }
-      }
-      cl.sync();
-      ++xk;
-      if (threadIdx.x > q && threadIdx.x < w) {
-        sig[threadIdx.x] = mine2->a[0][threadIdx.x] + mine2->a[1][threadIdx.x];
-        alp[threadIdx.x] = mine2->b[threadIdx.x];
-      }
-      __syncthreads();
+      const int np = pick(keys[0]);
+      if (np == wp || (np < 0 && wp == 0)) send(0, np >= 0, key_of(n1));
     }
-  }
-  // 3. Gram matrix of the reflectors (partials of both CTAs) and T
-  auto vv = [&](int s2, int rl) -> double {  // v_s2 at this CTA's row r0 + rl
-    const int r = r0 + rl;
-    return (r < s2) ? 0.0 : (r == s2 ? 1.0 : P[static_cast<size_t>(s2) * ml + rl]);
-  };
-  {
-    double(*gpeer)[kNB + 1] = cl.map_shared_rank(Gp[rank], peer);
-    // four pairs (s0 .. s0 + 3, q) per warp task, one butterfly for the four
-    // sums; only the tasks with s0 < q are enumerated (q = 1 .. w - 1 has
-    // ceil(q / 4) of them), so that the warps share them evenly
-    int ntask = 0;
-    for (int q = 1; q < w; ++q) ntask += (q + 3) / 4;
-    for (int task = wp; task < ntask; task += nw) {
-      int q = 1, rest = task;
-      while (rest >= (q + 3) / 4) {
-        rest -= (q + 3) / 4;
-        ++q;
-      }
-      const int s0 = 4 * rest;
-      double acc[4] = {0.0, 0.0, 0.0, 0.0};
-      for (int rl = lane; rl < ml; rl += 32) {
-        const double vq = vv(q, rl);
+    for (int j = 0; j < w; ++j) {
+      cl.sync();
+      int win = 0;
+      QbCand best = cand[j & 1][0];
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (s0 + u < q) acc[u] = fma(vv(s0 + u, rl), vq, acc[u]);
-      }
-      qb_wsum4(acc);
-      if (lane == 0)
-        for (int u = 0; u < 4 && s0 + u < q; ++u) {
-          Gp[rank][s0 + u][q] = acc[u];
-          gpeer[s0 + u][q] = acc[u];
+      for (int q = 1; q < kPCS; ++q) {
+        const QbCand y = cand[j & 1][q];
+        if (y.key > best.key || (y.key == best.key && y.col < best.col)) {
+          best = y;
+          win = q;
         }
+      }
+      const bool own = best.col == cid;
+      const double* xp = buf + ((j & 1) * kPCS + win) * mp + lane;
+      double v[kR];
+#pragma unroll
+      for (int t = 0; t < kR; ++t) v[t] = (t < nt) ? xp[32 * t] : 0.0;
+      if (lane <= j) v[0] = 0.0;
+      double a = 0.0;
+      if (exists && !own) {
+        a = x[0] * v[0];
+#pragma unroll
+        for (int t = 1; t < kR; ++t)
+          if (t < nt) a = fma(x[t], v[t], a);
+        a = qs_warp_sum(a);
+      }
+      const double xj = __shfl_sync(0xFFFFFFFFu, x[0], j);
+      qb_bar(1, 32 * (kPCW + 1));
+      const double vj = vj_sh;
+      double c = 0.0;
+      int rc = 0;
+      unsigned k = 0u;
+      if (own) {
+        step = j;
+        es = qb_exp(vj);
+        live = false;
+        if (lane == j) x[0] = vj;
+      } else if (exists) {
+        const double g = fma(vj, xj, a);
+        if (live) {
+          c = kap_sh * g;
+          const double rj = fma(-c, vj, xj);
+          if (lane == j) x[0] = rj;
+          n1 = fma(-rj, rj, n1);
+          if (__double2hiint(n1) < 0) n1 = 0.0;
+          const int hn = __double2hiint(n1), hr = __double2hiint(n2);
+          rc = (hn > hr - (26 << 20)) ? 0 : (hn > hr - (40 << 20)) ? 1 : 2;
+          k = key_of(n1);
+        } else if (lane < kPCS) {
+          *cl.map_shared_rank(&G[step][j], lane) = qb_shift(g, es + qb_exp(vj));
+        }
+      }
+      if (j + 1 == w) break;
+      if (lane == 0) {
+        keys[0][wp] = k;
+        wait_sum[wp] = rc == 2;
+      }
+      qb_bar(2, 32 * kPCW);
+      int np = pick(keys[0]);
+      const bool ahead = !__any_sync(0xFFFFFFFFu, lane < kPCW && wait_sum[lane]);
+      if (live) {
+#pragma unroll
+        for (int t = 0; t < kR; ++t)
+          if (t < nt) x[t] = fma(-c, v[t], x[t]);
+      }
+      if (!ahead) {
+        if (rc == 2) {
+          n1 = n2 = qs_warp_sum_pos(sumsq(j));
+          k = key_of(n1);
+        }
+        if (lane == 0) keys[1][wp] = k;
+        qb_bar(2, 32 * kPCW);
+        np = pick(keys[1]);
+      }
+      if (np == wp || (np < 0 && wp == 0))
+        send(j + 1, np >= 0, k);
+      else if (rc == 1)
+        n1 = n2 = qs_warp_sum_pos(sumsq(j));
     }
-  }
-  cl.sync();  // no shared memory of the peer is touched after this point
-  for (int e = threadIdx.x; e < w * w; e += blockDim.x) {  // Gp[0] <- V^T V (s < q)
-    const int s2 = e / w, q2 = e - s2 * w;
-    if (s2 < q2) Gp[0][s2][q2] += Gp[1][s2][q2];
-  }
-  __syncthreads();
-  if (wp == 0) {  // lanes over the rows i < q; four partial sums shorten the chain
-    auto gm = [&](int s2, int q2) -> double { return Gp[0][s2][q2]; };
-    for (int q = 0; q < w; ++q) {
-      const double tq = taus[q];
+    cl.sync();  // the Gram matrix is complete; no shared memory of a peer is touched any more
+  } else if (wp == kPCW) {
+    // column q of T from the Gram matrix; lanes over its rows, four partial
+    // sums shorten the chain
+    auto t_column = [&](int q) {
       double ti = 0.0;
       if (lane < q) {
-        double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-        for (int j = lane; j < q; j += 4) {
-          a0 = fma(T[lane][j], gm(j, q), a0);
-          if (j + 1 < q) a1 = fma(T[lane][j + 1], gm(j + 1, q), a1);
-          if (j + 2 < q) a2 = fma(T[lane][j + 2], gm(j + 2, q), a2);
-          if (j + 3 < q) a3 = fma(T[lane][j + 3], gm(j + 3, q), a3);
-        }
-        ti = -tq * ((a0 + a1) + (a2 + a3));
+        double a[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int i = lane; i < q; i += 4)
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            if (i + u < q) a[u] = fma(T[lane][i + u], G[i + u][q], a[u]);
+        ti = -kaps[q] * ((a[0] + a[1]) + (a[2] + a[3]));
       }
       __syncwarp();
-      if (lane < q) T[lane][q] = ti;
-      if (lane == 0) T[q][q] = tq;
-      for (int i = q + 1 + lane; i < w; i += 32) T[i][q] = 0.0;
+      T[lane][q] = (lane == q) ? kaps[q] : ti;
       __syncwarp();
+    };
+    for (int j = 0; j < w; ++j) {
+      cl.sync();
+      int win = 0;
+      QbCand best = cand[j & 1][0];
+#pragma unroll
+      for (int q = 1; q < kPCS; ++q) {
+        const QbCand y = cand[j & 1][q];
+        if (y.key > best.key || (y.key == best.key && y.col < best.col)) {
+          best = y;
+          win = q;
+        }
+      }
+      double beta, kap, vj;
+      qs_reflector(buf[((j & 1) * kPCS + win) * mp + j], best.sigma, beta, kap, vj);
+      if (lane == 0) {
+        kap_sh = kap;
+        vj_sh = vj;
+        betas[j] = beta;
+        vjs[j] = vj;
+        kaps[j] = qb_shift(kap, -2 * qb_exp(vj));
+      }
+      qb_bar(1, 32 * (kPCW + 1));
+      if (j > 0) t_column(j - 1);
+    }
+    cl.sync();
+    t_column(w - 1);
+  } else if (wp == kPCW + 1) {  // keeps the reflectors
+    if (rank == 0)
+      for (int pos = w + lane; pos < m; pos += 32) perm[c0 + pos] = pold[src_of[pos]];
+    for (int j = 0; j < w; ++j) {
+      cl.sync();
+      int win = 0;
+      QbCand best = cand[j & 1][0];
+#pragma unroll
+      for (int q = 1; q < kPCS; ++q) {
+        const QbCand y = cand[j & 1][q];
+        if (y.key > best.key || (y.key == best.key && y.col < best.col)) {
+          best = y;
+          win = q;
+        }
+      }
+      const double* xp = buf + ((j & 1) * kPCS + win) * mp + lane;
+      for (int t = 0; t < nt; ++t) Vb[j * mp + lane + 32 * t] = xp[32 * t];
+    }
+    cl.sync();
+  } else {
+    // whole rows of the trailing columns, one per warp and two steps; nothing
+    // here is shared, so the arrivals need not order it
+    constexpr int kSpare = kPW - kPCW - 2;
+    int pos = w + rank + kPCS * (wp - kPCW - 2);
+    double t[kR];
+    auto load = [&] {
+      const double* s = Ws + static_cast<size_t>(c0 + src_of[pos]) * n;
+#pragma unroll
+      for (int u = 0; u < kR; ++u) t[u] = (lane + 32 * u < n) ? s[lane + 32 * u] : 0.0;
+    };
+    auto store = [&] {
+      double* d = Wd + static_cast<size_t>(c0 + pos) * n;
+#pragma unroll
+      for (int u = 0; u < kR; ++u)
+        if (lane + 32 * u < n) d[lane + 32 * u] = t[u];
+      pos += kPCS * kSpare;
+    };
+    for (int j = 0; j <= w; ++j) {  // the w steps and the last barrier
+      if (pos < m) {
+        if (j & 1)
+          store();
+        else if (j < w)
+          load();
+      }
+      asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+      asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
+    while (pos < m) {
+      load();
+      store();
     }
   }
   __syncthreads();
-  // 4. outputs (this CTA's rows)
-  for (int e = threadIdx.x; e < w * ml; e += blockDim.x) {
-    const int q = e / ml, rl = e - q * ml, r = r0 + rl;
-    double y = 0.0;
-    for (int s2 = 0; s2 <= q; ++s2) y = fma(T[s2][q], vv(s2, rl), y);
-    Yt[static_cast<size_t>(c0 + q) * n + c0 + r] = y;
-    Vt[static_cast<size_t>(c0 + q) * n + c0 + r] = vv(q, rl);
-    Wd[static_cast<size_t>(c0 + q) * n + c0 + r] = (r == q) ? betas[q] : P[e];
+  // 3. V scaled; Y = T^T V^T
+  for (int q = wp; q < w; q += kPW) {
+    const double vj = vjs[q];
+    const int e = qb_exp(vj);
+    for (int r = lane; r < mp; r += 32)
+      Vb[q * mp + r] = (r < q) ? 0.0 : qb_shift(r == q ? vj : Vb[q * mp + r], e);
   }
-  for (int e = threadIdx.x + rank * blockDim.x; e < w * c0; e += 2 * blockDim.x) {
-    const int q = e / c0, r = e - q * c0;  // entries above the panel
-    Wd[static_cast<size_t>(c0 + q) * n + r] = Ws[static_cast<size_t>(c0 + src_of[lp[q]]) * n + r];
-  }
-  if (rank == 0 && threadIdx.x < w) {
-    const int q = threadIdx.x;
-    perm[c0 + q] = pold[src_of[lp[q]]];
-    double d = absd(betas[q]);
-    if (!(d > 0.0) || !isfinite(d)) {
-      atomicExch(status, d > 0.0 ? kDevNonFinite : kDevSingular);
-      if (!(d > 0.0)) d = DBL_MIN;
+  __syncthreads();
+  for (int g = rank; g < nt; g += kPCS) {
+    // a warp takes the columns i and 31 - i: 33 terms each
+    const int r = 32 * g + lane;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int q = h ? kNB - 1 - wp : wp;
+      if (q < w) {
+        double y0 = 0.0, y1 = 0.0;
+        int s = 0;
+        for (; s + 1 <= q; s += 2) {
+          y0 = fma(T[s][q], Vb[s * mp + r], y0);
+          y1 = fma(T[s + 1][q], Vb[(s + 1) * mp + r], y1);
+        }
+        if (s == q) y0 = fma(T[s][q], Vb[s * mp + r], y0);
+        if (r < m) {
+          Yt[static_cast<size_t>(c0 + q) * n + c0 + r] = y0 + y1;
+          Vt[static_cast<size_t>(c0 + q) * n + c0 + r] = Vb[q * mp + r];
+        }
+      }
     }
-    D[c0 + q] = d;
+  }
+  // 4. panel rows of this CTA's columns
+  if (wp < kPCW && cid < w) {
+    const int q = step;
+    double* d = Wd + static_cast<size_t>(c0 + q) * n;
+    const double* s = Ws + static_cast<size_t>(c0 + src_of[cid]) * n;
+    if (lane <= q) d[c0 + lane] = (lane == q) ? betas[q] : x[0];
+    for (int r = lane; r < c0; r += 32) d[r] = s[r];  // entries above the panel
+    if (lane == 0) {
+      perm[c0 + q] = pold[src_of[cid]];
+      double dd = absd(betas[q]);
+      if (!(dd > 0.0) || !isfinite(dd)) {
+        atomicExch(status, dd > 0.0 ? kDevNonFinite : kDevSingular);
+        if (!(dd > 0.0)) dd = DBL_MIN;
+      }
+      D[c0 + q] = dd;
+    }
   }
 }
 
@@ -558,7 +543,10 @@ int qr_blocked_launches(int n, int batch, int oz_batch) {
   return 2 + panels + (4 * panels - 2) * chunks;
 }
 
-size_t qr_blocked_smem(int n) { return static_cast<size_t>(kNB) * qb_split(n, kNB) * sizeof(double); }
+// Dynamic shared memory of a panel of w columns, m rows.
+static size_t qb_panel_smem(int w, int m) {
+  return static_cast<size_t>(w + 2 * kPCS) * ((m + 31) / 32 * 32) * sizeof(double);
+}
 
 cudaError_t launch_qr_blocked(double* Xt, long long sX, double* Qt, long long sQ, double* D,
                               long long sD, double* Rtil, long long sR, const QrbWork& wk, int n,
@@ -571,7 +559,7 @@ cudaError_t launch_qr_blocked(double* Xt, long long sX, double* Qt, long long sQ
   double* Yt = Xt;    // Y = T^T V^T of every panel
   double* Wt = wk.Wt;
   const long long sWt = wk.sWt;
-  const int smem = static_cast<int>(qr_blocked_smem(n));
+  const int smem = static_cast<int>(qb_panel_smem(kNB, n));
   cudaError_t e = cudaFuncSetAttribute(k_qrb_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   for (int c0 = 0, p = 0; c0 < n; c0 += kNB, ++p) {
@@ -579,15 +567,15 @@ cudaError_t launch_qr_blocked(double* Xt, long long sX, double* Qt, long long sQ
     const double* src = (p == 0) ? Xt : ((p & 1) ? WA : WB);
     const long long sSrc = (p == 0) ? sX : sW;
     double* dst = (p & 1) ? WB : WA;
-    {  // one cluster of two CTAs per matrix
+    {  // one cluster per matrix
       cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3(2 * batch, 1, 1);
+      cfg.gridDim = dim3(kPCS * batch, 1, 1);
       cfg.blockDim = dim3(kPT, 1, 1);
-      cfg.dynamicSmemBytes = static_cast<size_t>(w) * qb_split(m, w) * sizeof(double);
+      cfg.dynamicSmemBytes = qb_panel_smem(w, m);
       cfg.stream = st;
       cudaLaunchAttribute attr[1];
       attr[0].id = cudaLaunchAttributeClusterDimension;
-      attr[0].val.clusterDim.x = 2;
+      attr[0].val.clusterDim.x = kPCS;
       attr[0].val.clusterDim.y = 1;
       attr[0].val.clusterDim.z = 1;
       cfg.attrs = attr;

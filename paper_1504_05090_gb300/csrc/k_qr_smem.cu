@@ -44,6 +44,7 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "qr_scalars.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -64,87 +65,6 @@ __host__ __device__ __forceinline__ int qs_cols(int n, int cs) { return (n + cs 
 size_t qs_smem(int n, int cs) {
   const size_t ld = qs_ld(n);
   return (qs_cols(n, cs) * ld + (cs > 1 ? 2 * cs * ld : 0)) * sizeof(double);
-}
-
-// x 2^e for a normal x and a normal result, in the exponent field.
-__device__ __forceinline__ double qs_scale2(double x, int e) {
-  return __longlong_as_double(__double_as_longlong(x) + (static_cast<long long>(e) << 52));
-}
-
-// The leading 24 bits of a double in [1, 4) as a float, and a float as a
-// double, in integer arithmetic (a conversion would take the FP64 pipe).
-__device__ __forceinline__ float qs_to_f(double x) {
-  return __int_as_float(static_cast<int>((__double_as_longlong(x) >> 29) - (896LL << 23)));
-}
-__device__ __forceinline__ double qs_to_d(float x) {
-  return __longlong_as_double((static_cast<long long>(__float_as_int(x)) << 29) + (896LL << 52));
-}
-
-// Scalars of the reflector of (alpha, x), sigma = |x|^2 (see above): beta,
-// vj = v[j] and kap = 1 / (s u) = 1 / (n2 + |alpha| s), n2 = alpha^2 + sigma.
-// The square root and the reciprocal start from the FP32 approximations and
-// take one third-order Householder iteration each (relative error e of the
-// start, e^3 of the result): ten dependent FP64 instructions instead of the
-// thirty of sqrt() and a division.
-__device__ __forceinline__ void qs_reflector(double alpha, double sigma, double& beta, double& kap,
-                                             double& vj) {
-  beta = alpha;
-  kap = 0.0;
-  vj = 0.0;
-  if (__double_as_longlong(sigma) == 0LL) return;
-  const double n2 = fma(alpha, alpha, sigma), aa = absd(alpha);
-  const int E = static_cast<int>((__double_as_longlong(n2) >> 52) & 0x7FF);
-  double s;
-  if (E > 8 && E < 2036) {
-    const int e = (E - 1023) & ~1;            // n2 = m 2^e, m in [1, 4)
-    const double m = qs_scale2(n2, -e);
-    const double y0 = qs_to_d(rsqrtf(qs_to_f(m)));
-    const double t = m * y0;                  // about sqrt(m)
-    const double e1 = fma(-t, y0, 1.0);
-    const double q = e1 * fma(e1, 0.375, 0.5);
-    s = qs_scale2(fma(t, q, t), e / 2);
-    const double su = fma(aa, s, n2);         // in [n2, 2 n2]
-    const int eu = static_cast<int>((__double_as_longlong(su) >> 52) & 0x7FF) - 1023;
-    const double mu = qs_scale2(su, -eu);
-    const double r0 = qs_to_d(__fdividef(1.0f, qs_to_f(mu)));
-    const double e2 = fma(-mu, r0, 1.0);
-    kap = qs_scale2(fma(r0, fma(e2, e2, e2), r0), -eu);
-  } else {  // squares near the ends of the range (or not finite)
-    s = sqrt(n2);
-    kap = 1.0 / fma(aa, s, n2);
-  }
-  // comparisons on the sign bit (an FP64 one would take the FP64 pipe)
-  beta = (__double_as_longlong(alpha) < 0) ? s : -s;
-  vj = alpha - beta;
-}
-
-// Warp sum of non-negative finite numbers in 64-bit fixed point: aligned to
-// the largest exponent (58 bits, rounded), three integer warp reductions
-// instead of five rounds of shuffles and FP64 additions (about 130 against 650
-// clocks).  Error below 2^-53 of the sum.  Non-finite input gives non-finite
-// output.
-__device__ __forceinline__ double qs_warp_sum_pos(double a) {
-  const unsigned long long bits = static_cast<unsigned long long>(__double_as_longlong(a));
-  const int E = static_cast<int>((bits >> 52) & 0x7FF);
-  const int Emax = static_cast<int>(__reduce_max_sync(0xFFFFFFFFu, static_cast<unsigned>(E)));
-  if (Emax == 0x7FF) return __longlong_as_double(0x7FF8000000000000LL);
-  unsigned long long f = 0ull;
-  const int sh = Emax - E;
-  if (E != 0 && sh < 59) {
-    f = ((bits & ((1ull << 52) - 1)) | (1ull << 52)) << 5;
-    f = (f + ((1ull << sh) >> 1)) >> sh;
-  }
-  const unsigned l0 = static_cast<unsigned>(f) & 0x3FFFFFu, l1 = static_cast<unsigned>(f >> 22) & 0x3FFFFFu,
-                 l2 = static_cast<unsigned>(f >> 44);
-  const unsigned long long s = static_cast<unsigned long long>(__reduce_add_sync(0xFFFFFFFFu, l0)) +
-                               (static_cast<unsigned long long>(__reduce_add_sync(0xFFFFFFFFu, l1)) << 22) +
-                               (static_cast<unsigned long long>(__reduce_add_sync(0xFFFFFFFFu, l2)) << 44);
-  if (s == 0ull) return 0.0;
-  // s 2^(Emax - 1023 - 57); s in [2^57, 2^63)
-  const double d = __ull2double_rn(s);
-  const int e = Emax - 1023 - 57;
-  if (Emax > 64) return __longlong_as_double(__double_as_longlong(d) + (static_cast<long long>(e) << 52));
-  return ldexp(d, e);
 }
 
 // Sum over the kL lanes of a column.
