@@ -319,10 +319,7 @@ GemmArgs gemm0(int n) {
 // N >= kOzakiMinN unless the context asks for the FP64 pipe.
 cudaError_t gemm(dqmc_ctx* ctx, Group& g, const GemmArgs& m, int batch) {
   if (ctx->gemm_mode == DQMC_GEMM_TENSOR && g.oz) {
-    // the split and the MMA kernel (plus the balance pass) per chunk of the
-    // batch (the square products take the split path)
-    const int chunks = (batch + g.oz_batch - 1) / g.oz_batch;
-    ctx->launches += static_cast<long long>(chunks) * (m.balance ? 3 : 2) - 1;
+    ctx->launches += gemm_ozaki_launches(m, batch, g.oz_batch) - 1;
     return launch_gemm_ozaki(m, batch, g.oz, g.oz_batch, ctx->d_status, g.st);
   }
   return launch_gemm(m, batch, g.st);
