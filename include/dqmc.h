@@ -142,8 +142,11 @@ int dqmc_autotune(const dqmc_group* groups, int n_groups, double drift_target, u
  *               propagation of FP64 groups, gradient): 1, 2, 4, 8 or 16
  *               (<= N); 0 = built-in (4)
  *   wrap_nv     vectors per CTA of the slice wrap B_l G B_l^{-1} in the
- *               working precision (float-pair groups propagate G(tau) with
- *               twice as many): same values; 0 = built-in
+ *               working precision (float-pair groups off the tensor cores
+ *               propagate G(tau) with twice as many): same values; 0 =
+ *               built-in.  Of no effect on the wrap where one CTA takes a
+ *               matrix (N <= 24, or N <= 64 in float pairs or FP32 with at
+ *               least a chain per SM)
  *   metro_ctas  CTAs per chain of the Metropolis pass, one thread-block
  *               cluster (as dqmc_set_metropolis_split, for this group): 1, 2
  *               or 4 (4 * metro_ctas <= N); 0 = the context's setting */

@@ -308,6 +308,18 @@ int wrap_nv(const Group& g) {
   return std::min(4, g.N);
 }
 
+// The slice wrap as one launch with G in shared memory (k_wrap_smem; the same
+// numbers bit for bit, so the batch may decide).  Two passes spread one matrix
+// over N / 4 CTAs each and win while the chip has SMs to spare: 8 x 8 FP32, 32
+// chains 8.1 + 8.1 us against 16.2; 256 chains in float pairs 37.7 + 37.7 against
+// 38.5 (three groups side by side).  At N <= 24 a launch is all there is: 4 x 4,
+// one chain 8.0 + 8.0 against 8.9.  Larger FP64 matrices are bound by the FP64
+// pipe either way (67 us a pass for 512 of 8 x 8, all of it multiply-adds).
+template <typename T>
+bool wrap_on_chip(int N, int chains, int nsm) {
+  return N <= 24 || (!std::is_same<T, double>::value && N <= 64 && chains >= nsm);
+}
+
 GemmArgs gemm0(int n) {
   GemmArgs a{};
   a.n = n;
@@ -564,10 +576,15 @@ int up_pass(dqmc_ctx* ctx, Group& g, int measure) {
     DQ_CLASS(ctx, kTMetropolis);
     DQ_LAUNCH(ctx, launch_metropolis<T>(Gw, g.field, g.C, ma, g.st));
     wl.l0_first = wr.l0_first = l - 1;
-    DQ_CLASS(ctx, kTWrap);
-    DQ_LAUNCH(ctx, launch_kron_cols<T>(Gw, g.C, wl, g.st));
-    DQ_CLASS(ctx, kTWrap);
-    DQ_LAUNCH(ctx, launch_kron_rows<T>(Gw, Gw, g.C, wr, g.st));
+    if (wrap_on_chip<T>(g.N, g.C, ctx->nsm)) {
+      DQ_CLASS(ctx, kTWrap);
+      DQ_LAUNCH(ctx, launch_wrap_smem<T>(Gw, g.C, wl, g.st));
+    } else {
+      DQ_CLASS(ctx, kTWrap);
+      DQ_LAUNCH(ctx, launch_kron_cols<T>(Gw, g.C, wl, g.st));
+      DQ_CLASS(ctx, kTWrap);
+      DQ_LAUNCH(ctx, launch_kron_rows<T>(Gw, Gw, g.C, wr, g.st));
+    }
     if (l == g.cp[j]) {
       DQ_RET(stack_right(ctx, g, j));
       DQ_RET(recompute(ctx, g, j));

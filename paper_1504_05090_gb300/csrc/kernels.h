@@ -82,6 +82,10 @@ template <typename T>
 cudaError_t launch_metropolis(T* G, int8_t* field, int C, const MetroArgs& a, cudaStream_t st);
 template <typename T>
 cudaError_t launch_kron_rows(const T* in, T* out, int batch, const KronArgs& a, cudaStream_t st);
+// Both passes of a slice wrap in one launch, G in shared memory (N <= 64; a:
+// the arguments of the columns' pass).  Same result bit for bit.
+template <typename T>
+cudaError_t launch_wrap_smem(T* X, int batch, const KronArgs& a, cudaStream_t st);
 template <typename T>
 cudaError_t launch_kron_cols(T* X, int batch, const KronArgs& a, cudaStream_t st);
 template <typename T>
