@@ -288,14 +288,13 @@ def class_work(cls, acceptance, precision):
         return "alu32x2", C * (nc + 1) * g3
     if cls in ("stack_kron", "gtau_propagate"):
         # two matrices (right and left stack; G(l,0) and Y) x L slices x N vectors
-        # x 2N(Lx+Ly) flops per Kronecker application.  The stack products (and
-        # the G(tau) propagation of FP64 groups) run on the tensor cores as 36
-        # BF16 digit products per FP64 product; float-pair groups propagate
-        # G(tau) in float pairs on the FP32 pipe
+        # x 2N(Lx+Ly) flops per Kronecker application, on the tensor cores as 28
+        # BF16 digit products per FP64 product; float-pair groups of small
+        # lattices propagate G(tau) in float pairs on the FP32 pipe
         fp64eq = C * 2 * L * N * 2 * N * (Lx + Ly)
-        if cls == "gtau_propagate" and precision == "df32":
+        if cls == "gtau_propagate" and precision == "df32" and Lx + Ly < 28:
             return "alu32x2", fp64eq
-        return "tensor", 36 * fp64eq
+        return "tensor", 28 * fp64eq
     if cls == "metropolis":  # rank-1 Sherman-Morrison update per accepted flip
         return ("alu32x2" if precision == "df32" else "alu"), acceptance * C * N * L * 2.0 * N * N
     if cls == "wrap":  # B G B^-1 by Kronecker factors: 2 sides x N vectors x 2N(Lx+Ly)
