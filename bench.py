@@ -672,7 +672,7 @@ def run_config(args):
 def bench_config():
     """The workload description both arms report."""
     return {"workload": WORKLOAD, "precision": "df32 (float pairs) Metropolis/delayed "
-            "update/wrap/G(tau) propagation, fp64 UDV/QR stabilisation, G recompute, drift",
+            "update/wrap, fp64 UDV/QR stabilisation, G recompute, G(tau) propagation, drift",
             "chains_per_gpu": W["chains"], "L2": "working set > L2 (no flush needed)"}
 
 
