@@ -791,6 +791,67 @@ struct alignas(2 * sizeof(T)) KronPair {
   T a, b;
 };
 
+// Tap t of a table (below).  Float pairs on even sides: taps 2i, 2i + 1 as
+// (hi, hi, lo, lo), so that one 16-byte load gives both packed operands.
+template <typename T>
+__device__ __forceinline__ void kron_put_tap(T* tab, int t, double x, bool even) {
+  if constexpr (std::is_same<T, df32>::value) {
+    if (even) {
+      const df32 d(x);
+      float* f = reinterpret_cast<float*>(tab) + 4 * (t >> 1) + (t & 1);
+      f[0] = d.hi;
+      f[2] = d.lo;
+      return;
+    }
+  }
+  tab[t] = static_cast<T>(x);
+}
+
+// One side of the transform in float pairs, both sides even: two neighbouring
+// outputs along the side are the two lanes of packed sums, and a thread takes
+// them for V vectors (vi, vi + nv / V), which share the tap load.  The same
+// operations in the same order per output as with scalar sums.
+// What bounds it: issue slots and the latency of the loads; a term's twelve
+// packed operations stand for 24 scalar ones, which leaves slots for the loads.
+// Two vectors per thread where that still gives every thread of the CTA work
+// (nv N >= 4 threads: 4 vectors at 16 x 16, all of 8 x 8 in one CTA), else one.
+// Sweeps with scalar sums, then packed: 16 x 16, 64 chains 379.4 -> 375.7 ms
+// (320 passes, 11 us each); 8 x 8, 3 x 256 chains 117.4 -> 115.7; two chains of
+// 16 x 16 unchanged at 80.1.
+template <int V, bool kY>
+__device__ __forceinline__ void kron_side_df32(const df32* in, df32* out, int nv, int ld, int Lx,
+                                               int Ly, const df32* t0, const df32* t1,
+                                               const df32* post) {
+  const int h = nv / V, per = (Lx * Ly) >> 1, n = kY ? Ly : Lx, w = kY ? Lx : Lx >> 1;
+  const int str = kY ? Lx : 1;
+  for (int e = threadIdx.x; e < h * per; e += blockDim.x) {
+    const int vi = e / per, rr = e - vi * per, q = rr / w, r = rr - q * w;
+    const int o = 2 * (kY ? q : r);  // the first output along the side
+    const int base = vi * ld + (kY ? r : Lx * q);
+    const df32* p = in + base;
+    ProdSum2 a[V];
+#pragma unroll 2
+    for (int k = 0; k < n; ++k) {
+      const int b = o + n - k;  // tap index of output o; b + 1 that of o + 1
+      const ulonglong2 t = *reinterpret_cast<const ulonglong2*>((b & 1) ? t1 + b - 1 : t0 + b);
+#pragma unroll
+      for (int u = 0; u < V; ++u) {
+        const df32 x = p[u * h * ld + str * k];
+        a[u].add(t.x, t.y, pk_pack(x.hi, x.hi), pk_pack(x.lo, x.lo), pk_pack(-x.hi, -x.hi));
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < V; ++u) {
+      df32 y0, y1;
+      a[u].get(y0, y1);
+      const int i0 = (kY ? r : Lx * q) + str * o, i1 = i0 + str;
+      df32* d = out + (vi + u * h) * ld;
+      d[i0] = post ? y0 * post[i0] : y0;
+      d[i1] = post ? y1 * post[i1] : y1;
+    }
+  }
+}
+
 template <typename T>
 __device__ __forceinline__ void kron_transform(T* v, T* tmp, int nv, int ld, int Lx, int Ly, int N,
                                                const T* tx, const T* ty, const T* txs,
@@ -809,6 +870,19 @@ __device__ __forceinline__ void kron_transform(T* v, T* tmp, int nv, int ld, int
     // entry (one load), and their taps E[x - x'], E[x + 1 - x'] are adjacent:
     // one 16-byte load from tx (tap index even) or from txs, the same taps
     // shifted by one (odd).  Same additions in the same order per output.
+    if constexpr (std::is_same<T, df32>::value) {
+      if ((nv & 1) == 0 && nv * N >= 4 * static_cast<int>(blockDim.x)) {
+        kron_side_df32<2, false>(v, tmp, nv, ld, Lx, Ly, tx, txs, nullptr);
+        __syncthreads();
+        kron_side_df32<2, true>(tmp, v, nv, ld, Lx, Ly, ty, tys, post);
+      } else {
+        kron_side_df32<1, false>(v, tmp, nv, ld, Lx, Ly, tx, txs, nullptr);
+        __syncthreads();
+        kron_side_df32<1, true>(tmp, v, nv, ld, Lx, Ly, ty, tys, post);
+      }
+      __syncthreads();
+      return;
+    }
     const int hx = Lx >> 1, hy = Ly >> 1;
     const int ptx = nv * Ly * hx;
     for (int e = threadIdx.x; e < ptx; e += blockDim.x) {
@@ -935,12 +1009,12 @@ template <typename T>
 __device__ __forceinline__ void kron_load_taps(const KronArgs& a, KronStage<T> s) {
   if (threadIdx.x < 2 * kMaxSide) {  // each circulant row twice over (kron_transform)
     const int t = threadIdx.x, tx = t % a.Lx, ty = t % a.Ly;
-    const bool inv = (a.kind == kBIT);
-    s.tx[t] = static_cast<T>(inv ? a.taps.exi[tx] : a.taps.ex[tx]);
-    s.ty[t] = static_cast<T>(inv ? a.taps.eyi[ty] : a.taps.ey[ty]);
+    const bool inv = (a.kind == kBIT), ev = ((a.Lx | a.Ly) & 1) == 0;
     const int tx1 = (t + 1) % a.Lx, ty1 = (t + 1) % a.Ly;
-    s.txs[t] = static_cast<T>(inv ? a.taps.exi[tx1] : a.taps.ex[tx1]);
-    s.tys[t] = static_cast<T>(inv ? a.taps.eyi[ty1] : a.taps.ey[ty1]);
+    kron_put_tap(s.tx, t, inv ? a.taps.exi[tx] : a.taps.ex[tx], ev);
+    kron_put_tap(s.ty, t, inv ? a.taps.eyi[ty] : a.taps.ey[ty], ev);
+    kron_put_tap(s.txs, t, inv ? a.taps.exi[tx1] : a.taps.ex[tx1], ev);
+    kron_put_tap(s.tys, t, inv ? a.taps.eyi[ty1] : a.taps.ey[ty1], ev);
   }
 }
 
@@ -1058,14 +1132,15 @@ __global__ void __launch_bounds__(kWT, 2) k_wrap_smem(T* X, KronArgs a) {
   }
   if (threadIdx.x < 2 * kMaxSide) {  // each circulant row twice over (kron_transform)
     const int t = threadIdx.x, tx = t % a.Lx, ty = t % a.Ly, tx1 = (t + 1) % a.Lx, ty1 = (t + 1) % a.Ly;
-    s.tx[t] = static_cast<T>(a.taps.ex[tx]);
-    s.ty[t] = static_cast<T>(a.taps.ey[ty]);
-    s.txs[t] = static_cast<T>(a.taps.ex[tx1]);
-    s.tys[t] = static_cast<T>(a.taps.ey[ty1]);
-    taps2[t] = static_cast<T>(a.taps.exi[tx]);
-    taps2[2 * kMaxSide + t] = static_cast<T>(a.taps.eyi[ty]);
-    taps2[4 * kMaxSide + t] = static_cast<T>(a.taps.exi[tx1]);
-    taps2[6 * kMaxSide + t] = static_cast<T>(a.taps.eyi[ty1]);
+    const bool ev = ((a.Lx | a.Ly) & 1) == 0;
+    kron_put_tap(s.tx, t, a.taps.ex[tx], ev);
+    kron_put_tap(s.ty, t, a.taps.ey[ty], ev);
+    kron_put_tap(s.txs, t, a.taps.ex[tx1], ev);
+    kron_put_tap(s.tys, t, a.taps.ey[ty1], ev);
+    kron_put_tap(taps2, t, a.taps.exi[tx], ev);
+    kron_put_tap(taps2 + 2 * kMaxSide, t, a.taps.eyi[ty], ev);
+    kron_put_tap(taps2 + 4 * kMaxSide, t, a.taps.exi[tx1], ev);
+    kron_put_tap(taps2 + 6 * kMaxSide, t, a.taps.eyi[ty1], ev);
   }
   const T up = static_cast<T>(a.ec), dn = static_cast<T>(a.emc);
   const int8_t* f = a.field + (static_cast<size_t>(b) * a.L + a.l0_first) * N;
