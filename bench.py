@@ -235,7 +235,7 @@ DF32_PEAK = 2 * 152 * 128 * 2.07e9 / 14 / 1e12
 TRAFFIC = {
     # panel x 8, fused rank-32 products x 30, finalize: one blocked QR launch
     ("qr_pivot", None): (687.3e6, ("k_qr_blocked.cu", "k_ozaki.cu"), "443fe89b26ebd644"),
-    ("metropolis", "df32"): (33.67e6, ("k_sweep.cu",), "3397bbe4cabbe44d"),
+    ("metropolis", "df32"): (33.67e6, ("k_sweep.cu",), "a31adbbee642dc65"),
     ("stack_kron", None): (34.09e6, ("k_kron_tc.cu",), "33ed7cfa2a480480"),
 }
 

@@ -811,8 +811,10 @@ __device__ __forceinline__ void kron_put_tap(T* tab, int t, double x, bool even)
 // outputs along the side are the two lanes of packed sums, and a thread takes
 // them for V vectors (vi, vi + nv / V), which share the tap load.  The same
 // operations in the same order per output as with scalar sums.
-// What bounds it: issue slots and the latency of the loads; a term's twelve
-// packed operations stand for 24 scalar ones, which leaves slots for the loads.
+// What bounds it: no one thing at 16 x 16 (issue slots 57 % busy; the waits are
+// shared by the FP32 pipe, dependent sums, loads of the tile and barriers).  A
+// term's twelve packed operations stand for 24 scalar ones and leave slots for
+// the loads.
 // Two vectors per thread where that still gives every thread of the CTA work
 // (nv N >= 4 threads: 4 vectors at 16 x 16, all of 8 x 8 in one CTA), else one.
 // Sweeps with scalar sums, then packed: 16 x 16, 64 chains 379.4 -> 375.7 ms
