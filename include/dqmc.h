@@ -189,8 +189,11 @@ int dqmc_recompute_G(dqmc_ctx* ctx, double* max_drift_out);
  * with index kx + Lx*ky.  G(l,0) is formed stably (FP64) at every
  * stabilisation point and propagated by B_l in between: to FP64 accuracy, or
  * in float pairs (agreeing to about 1e-9 of the maximum) for groups with
- * DQMC_DF32 working precision with Lx + Ly < 28 or in DQMC_GEMM_FP64 mode.
- * Row length per chain is
+ * DQMC_DF32 working precision with Lx + Ly < 28, in DQMC_GEMM_FP64 mode or
+ * with a long interval.  An interval is long where 2 n_s (lambda + 4 |t| dtau)
+ * > 16, cosh(lambda) = e^{dtau U / 2}: whatever the precision, single entries
+ * of G(tau) then carry the rounding of a UDV stack step amplified (by 1e-8 to
+ * 1e-7 of the RMS at 22).  Row length per chain is
  * (L_g + 1) * N_g of its group; dqmc_gtau_size() gives the total.
  * out: caller-owned doubles, on the device if out_on_device else on the host.
  * Requires current UDV stacks (true after dqmc_init, dqmc_sweep,
@@ -365,6 +368,8 @@ int dqmc_set_gemm_mode(dqmc_ctx* ctx, int mode);
  *   DQMC_QR_PIVOTED: Householder QR with column pivoting on the FP64 pipe
  *     (always used for N <= 144, where the matrix stays in shared memory, and
  *     in DQMC_GEMM_FP64 mode).
+ * Groups with a long interval (dqmc_measure_Gtau) use the blocked QR from
+ * N = 64 on and the pivoted one, on global memory, below.
  * Both give X = U D T with |diag| T = 1; G agrees between them to the
  * conditioning of the problem.  Drops captured sweep graphs.  Errors:
  * DQMC_ERR_ARG. */

@@ -89,6 +89,7 @@ struct Group {
   dqmc_group p;
   int N = 0, L = 0, nc = 0, C = 0, chain0 = 0;
   double lam = 0.0;
+  bool long_step = false;  // see stretches_far
   std::vector<int> cp;
   KronTaps taps{};
   int8_t* field = nullptr;
@@ -172,6 +173,23 @@ namespace {
 constexpr int kOzakiMinN = 64;  // smaller matrices stay on the FP64 pipe
 constexpr double kTuneMargin = 0.05;  // probe drift must stay below 5% of the target
 
+// One factor B_l stretches a vector by at most e^{+-(lambda + 4 |t| dtau)}, so
+// the columns of a stack step over n slices spread by up to e^{2 n (lambda +
+// 4 |t| dtau)}, and the rounding of the step comes out of it amplified.  Two
+// FP64-accurate ways to form the stacks then give G(tau) that differ, in the
+// worst entry relative to its RMS (8 x 8, 128 chains; 10 x 10, 96), by
+//   exponent 12.7: 6e-12, 8e-12    13.7: 1e-11, 7e-11    17.2: 9e-10, 2e-9
+//            20.5: 6e-10, 2e-9     21.7: 1e-8, 1e-8 (7e-8 over more chains)
+// in FP64 and float-pair groups alike.  Beyond kLongStep such a difference is
+// no longer small, and it is as large against the exact value whichever way is
+// taken.  The groups there keep the kernels that their stacks have always been
+// formed by, operation for operation, so that G(tau) of a field is reproduced:
+// k_qrp_cluster (N < 64), panels of two CTAs and Kronecker products of eight
+// digits.  A common interval (n_s dtau = 1.25, U <= 3) has 12 to 15.
+constexpr double kLongStep = 16.0;
+bool stretches_far(const dqmc_group& p, int L, double lam) {
+  return 2.0 * std::min(p.stab_interval, L) * (lam + 4.0 * std::fabs(p.t) * p.dtau) > kLongStep;
+}
 
 #define DQ_CK(call)                                 \
   do {                                              \
@@ -281,6 +299,7 @@ KronArgs kron_base(const Group& g, int kind, int nv) {
   a.out_stride = g.nn();
   a.per_chain = 1;
   a.dir = 1;
+  a.digits8 = g.long_step;
   return a;
 }
 
@@ -339,19 +358,20 @@ cudaError_t gemm(dqmc_ctx* ctx, Group& g, const GemmArgs& m, int batch) {
 
 // QR of the stack step X = B..B (U D) (rows of g.X = columns of X) into the
 // stack entry (Q^T at Qt, D at Dv) and g.Rtil: column-pivoted with the matrix
-// in shared memory up to N = 144 (qr_smem_ctas), else the blocked QR with
-// tensor-core updates where the tensor-core products are in use, else the
-// column-pivoted cluster QR on global memory.
+// in shared memory up to N = 144 (qr_smem_ctas; not where a step stretches far,
+// see kLongStep), else the blocked QR with tensor-core updates where the
+// tensor-core products are in use, else the column-pivoted cluster QR on global
+// memory.
 cudaError_t stack_qr(dqmc_ctx* ctx, Group& g, double* Qt, double* Dv) {
   const long long sD = static_cast<long long>(g.nc + 1) * g.N;
-  const int cs = qr_smem_ctas(g.N, ctx->total, ctx->nsm);
+  const int cs = g.long_step ? 0 : qr_smem_ctas(g.N, ctx->total, ctx->nsm);
   if (cs > 0)
     return launch_qr_smem(cs, g.X, g.nn(), Qt, g.sstride(), Dv, sD, g.Rtil, g.nn(), g.N, g.C,
                           ctx->d_status, g.st);
   if (ctx->gemm_mode == DQMC_GEMM_TENSOR && ctx->qr_mode == DQMC_QR_BLOCKED && g.oz) {
     ctx->launches += qr_blocked_launches(g.N, g.C, g.oz_batch) - 1;
     return launch_qr_blocked(g.X, g.nn(), Qt, g.sstride(), Dv, sD, g.Rtil, g.nn(), g.qrb, g.N, g.C,
-                             g.oz, g.oz_batch, ctx->d_status, g.st);
+                             g.oz, g.oz_batch, ctx->d_status, g.st, g.long_step);
   }
   return launch_qrp_cluster(g.X, g.nn(), Qt, g.sstride(), Dv, sD, g.Rtil, g.nn(), g.qrs, g.N, g.C,
                             ctx->d_status, g.st);
@@ -713,6 +733,7 @@ int setup_group(dqmc_ctx* ctx, Group& g) {
   g.L = static_cast<int>(std::llround(p.beta / p.dtau));
   g.C = p.n_chains;
   g.lam = std::acosh(std::exp(0.5 * p.dtau * p.U));
+  g.long_step = stretches_far(p, g.L, g.lam);
   g.cp.clear();
   for (int j = 0;; ++j) {
     const int c = std::min(j * p.stab_interval, g.L);
@@ -1168,7 +1189,9 @@ int measure_gtau_group(dqmc_ctx* ctx, Group& g, double* dst) {
     // 16, the float-pair one works for Lx + Ly: 16 x 16, 64 chains, 17 points
     // 17.2 against 25.7 ms, 8 x 8, 768 chains 12.2 against 11.6 ms; by the work
     // of both per element they meet near 13 x 13.
-    const bool tc = ctx->gemm_mode == DQMC_GEMM_TENSOR && g.oz && (!pair || g.p.Lx + g.p.Ly >= 28);
+    const bool tc = ctx->gemm_mode == DQMC_GEMM_TENSOR && g.oz &&
+                    (!pair || (g.p.Lx + g.p.Ly >= 28 && !g.long_step));
+    ga.digits8 = g.long_step;
     ga.kind = kB; ga.vec_is_col = 1; ga.bin_slot = 0;
     DQ_CLASS(ctx, kTGtauProp);
     DQ_LAUNCH(ctx, tc ? launch_gtau_tc(g.A1, batch, ga, ctx->d_status, g.st)

@@ -29,15 +29,19 @@
 // find different banks.  One launch of the 16 x 16 sweep (64 chains x 256
 // vectors x 10 slices): 1.32 ms with eight 7-bit digits, FP64 conversions and
 // rows of Lx, 0.61 ms now.
-#include <cuda_bf16.h>
-
+//
+// Eight 7-bit digits (TcDigits8: 53 bits, truncated, 36 products, rounded once
+// from two 64-bit integers) stay for the groups whose stack steps stretch a
+// vector so far that single entries of G(tau) carry the rounding of a step
+// amplified to 1e-8 and more (long_step in dqmc.cu): their numbers depend on
+// every rounding and are kept as they are.
 #include "common.cuh"
 #include "kernels.h"
+#include "oz_compose.cuh"
 
 namespace dqmc {
 namespace {
 
-constexpr int kS = 7;       // digit slices
 constexpr int kR = 128;     // rows of one product (TMEM lanes)
 constexpr int kK = 16;      // inner dimension (padded side)
 constexpr int kTC = 128;    // threads
@@ -73,64 +77,142 @@ __device__ __forceinline__ bool tc_wait(uint64_t* bar, int parity) {
   return done != 0;
 }
 
-// Exponent to align a vector to: the largest biased exponent, one higher where
-// the leading seven bits of the significand are all ones, so that the top
-// digit of the aligned number, rounded up by the digits below it, stays below
-// 128.
-__device__ __forceinline__ int tc_exp(double x) {
-  return ((__double2hiint(x) & 0x7FFFFFFF) + 0x4000) >> 20;
-}
-
-// x as the integer round-down(|x| 2^(1077 - emax)) with x's sign, below 2^55,
-// plus 128 in each of its seven bytes: byte 6 - p is then digit p plus 128.
-__device__ __forceinline__ unsigned long long tc_align(double x, int emax) {
-  const long long bits = __double_as_longlong(x);
-  const int E = static_cast<int>((bits >> 52) & 0x7FF);
-  long long m = 0;
-  if (E != 0) {  // zero and subnormal inputs contribute zero digits
-    const unsigned long long mant =
-        ((static_cast<unsigned long long>(bits) & ((1ULL << 52) - 1)) | (1ULL << 52)) << 2;
-    const int sh = emax - E;
-    m = (sh < 64) ? static_cast<long long>(mant >> sh) : 0LL;
-    if (bits < 0) m = -m;
-  }
-  return static_cast<unsigned long long>(m) + 0x0080808080808080ULL;
-}
-
-// Digit p of an aligned number as a float: the byte in the low bits of 2^23,
-// minus 2^23 + 128.
-__device__ __forceinline__ float tc_digit(unsigned long long t, int p) {
-  const uint32_t w = (p < 3) ? static_cast<uint32_t>(t >> 32) : static_cast<uint32_t>(t);
-  const int byte = (p < 3) ? 2 - p : 6 - p;
-  return __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7440u | byte)) - 8388736.0f;
-}
-
 // Two floats with at most eight significant bits as a BF16 pair: their high
 // halves.
 __device__ __forceinline__ uint32_t tc_pack(float a, float b) {
   return __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
 }
 
+// The number W 2^(e - 2102), W the integer sum of the accumulators, rounded to
+// FP64 (W's leading 53 bits; e: the sum of the two biased exponents).
+__device__ __forceinline__ double tc_compose(long long W, int e) {
+  const unsigned long long x = static_cast<unsigned long long>(W < 0 ? -W : W);
+  const int lz = __clzll(static_cast<long long>(x));
+  const unsigned long long m = ((x << (lz - 1)) + 0x200u) >> 10;  // 2^52 .. 2^53
+  const int ef = e - 1016 - lz;
+  if (x != 0 && (ef < 1 || ef > 2045)) return ldexp(static_cast<double>(W), e - 2102);
+  unsigned long long r = (static_cast<unsigned long long>(ef - 1) << 52) + m;
+  if (W < 0) r |= 0x8000000000000000ULL;
+  return (x == 0) ? 0.0 : __longlong_as_double(static_cast<long long>(r));
+}
+
+// Seven balanced digits of eight bits.
+struct TcDigits7 {
+  static constexpr int kS = 7;  // digit slices
+
+  // Exponent to align a vector to: the largest biased exponent, one higher where
+  // the leading seven bits of the significand are all ones, so that the top
+  // digit of the aligned number, rounded up by the digits below it, stays below
+  // 128.
+  static __device__ __forceinline__ int expo(double x) {
+    return ((__double2hiint(x) & 0x7FFFFFFF) + 0x4000) >> 20;
+  }
+
+  // x as the integer round-down(|x| 2^(1077 - emax)) with x's sign, below 2^55,
+  // plus 128 in each of its seven bytes: byte 6 - p is then digit p plus 128.
+  static __device__ __forceinline__ unsigned long long align(double x, int emax) {
+    const long long bits = __double_as_longlong(x);
+    const int E = static_cast<int>((bits >> 52) & 0x7FF);
+    long long m = 0;
+    if (E != 0) {  // zero and subnormal inputs contribute zero digits
+      const unsigned long long mant =
+          ((static_cast<unsigned long long>(bits) & ((1ULL << 52) - 1)) | (1ULL << 52)) << 2;
+      const int sh = emax - E;
+      m = (sh < 64) ? static_cast<long long>(mant >> sh) : 0LL;
+      if (bits < 0) m = -m;
+    }
+    return static_cast<unsigned long long>(m) + 0x0080808080808080ULL;
+  }
+
+  // Digit p of an aligned number as a float: the byte in the low bits of 2^23,
+  // minus 2^23 + 128.
+  static __device__ __forceinline__ float digit(unsigned long long t, int p) {
+    const uint32_t w = (p < 3) ? static_cast<uint32_t>(t >> 32) : static_cast<uint32_t>(t);
+    const int byte = (p < 3) ? 2 - p : 6 - p;
+    return __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7440u | byte)) - 8388736.0f;
+  }
+
+  // The result from the accumulators P_d, integers below 2^21, read off the low
+  // bits of 1.5 2^23 + P_d (as P_d + kM): W = sum_d P_d 2^(44 - 8 d) (d = 6
+  // rounded), below 2^63; ea, eb: the exponents of the two operands.
+  static __device__ __forceinline__ double compose(const uint32_t (&acc)[kS], int ea, int eb) {
+    constexpr uint32_t kM = 0x4B400000u;
+    uint32_t u[kS];
+#pragma unroll
+    for (int d = 0; d < kS; ++d) u[d] = __float_as_uint(__uint_as_float(acc[d]) + 12582912.0f);
+    const int a = static_cast<int>(u[0] * 256u + u[1] - kM * 257u);
+    const int b = static_cast<int>(u[2] * 256u + u[3] - kM * 257u);
+    const int c = static_cast<int>(u[4] * 256u + u[5] - kM * 257u);
+    const int g = static_cast<int>(u[6] - kM);
+    const long long W = ((static_cast<long long>(a) * 65536 + b) << 20) +
+                        (static_cast<long long>(c) << 4) + ((g + 8) >> 4);
+    return tc_compose(W, ea + eb);
+  }
+};
+
+// Eight digits of seven bits (the last of four), of the magnitude with x's sign.
+struct TcDigits8 {
+  static constexpr int kS = 8;
+
+  static __device__ __forceinline__ int expo(double x) { return (__double2hiint(x) >> 20) & 0x7FF; }
+
+  // the significand shifted down to emax, x's sign on top
+  static __device__ __forceinline__ unsigned long long align(double x, int emax) {
+    const unsigned long long bits = static_cast<unsigned long long>(__double_as_longlong(x));
+    const int E = static_cast<int>((bits >> 52) & 0x7FF), sh = emax - E;
+    unsigned long long al = 0ULL;
+    if (E != 0 && sh < 64) al = ((bits & ((1ULL << 52) - 1)) | (1ULL << 52)) >> sh;
+    return al | (bits & 0x8000000000000000ULL);
+  }
+
+  static __device__ __forceinline__ float digit(unsigned long long t, int p) {
+    const uint32_t d = (p < 7) ? static_cast<uint32_t>(t >> (46 - 7 * p)) & 127u
+                               : (static_cast<uint32_t>(t) & 15u) << 3;
+    const uint32_t sign = static_cast<uint32_t>(t >> 32) & 0x80000000u;
+    return __uint_as_float(__float_as_uint(__uint_as_float(0x4B000000u | d) - 8388608.0f) | sign);
+  }
+
+  // (hi + 2^-28 lo) 2^{e - 21} with e the sum of the operands' exponents less
+  // 6 each, rounded once (FP64 products where it leaves the normal range)
+  static __device__ __forceinline__ double compose(const uint32_t (&acc)[kS], int ea, int eb) {
+    int n[kS];
+#pragma unroll
+    for (int d = 0; d < kS; ++d)
+      n[d] = __float_as_int(__uint_as_float(acc[d]) + 12582912.0f) - 0x4B400000;
+    long long hi = 0, lo = 0;
+#pragma unroll
+    for (int d = 0; d < 4; ++d) hi += static_cast<long long>(n[d]) * (1 << (7 * (3 - d)));
+#pragma unroll
+    for (int d = 4; d < kS; ++d) lo += static_cast<long long>(n[d]) * (1 << (7 * (7 - d)));
+    const int fa = ea - 1029, fb = eb - 1029 - 21;
+    bool ok;
+    const double v = oz_compose(hi, lo, fa + fb, false, ok);
+    if (ok) return v;
+    return fma(static_cast<double>(lo), 0x1p-28, static_cast<double>(hi)) * ldexp(1.0, fa) * ldexp(1.0, fb);
+  }
+};
+
 // Digits of the taps as the right operand: column j, inner index k,
 // t[(j - k) mod n] for j, k < n (zero padding beyond); the columns hold the same
 // taps, so they share one exponent, which is returned.
+template <class Dg>
 __device__ int tc_tap_digits(const double* t, int n, unsigned char* bs) {
   int emax = 0;
-  for (int k = 0; k < n; ++k) emax = max(emax, tc_exp(t[k]));
+  for (int k = 0; k < n; ++k) emax = max(emax, Dg::expo(t[k]));
   for (int e = threadIdx.x; e < kK * kK; e += blockDim.x) {
     const int j = e / kK, k = e - j * kK;
-    const unsigned long long v = tc_align((j < n && k < n) ? t[(j - k + n) % n] : 0.0, emax);
-    for (int p = 0; p < kS; ++p)
+    const unsigned long long v = Dg::align((j < n && k < n) ? t[(j - k + n) % n] : 0.0, emax);
+    for (int p = 0; p < Dg::kS; ++p)
       reinterpret_cast<uint16_t*>(bs + p * kBSlice)[tc_off(j, k)] =
-          static_cast<uint16_t>(__float_as_uint(tc_digit(v, p)) >> 16);
+          static_cast<uint16_t>(__float_as_uint(Dg::digit(v, p)) >> 16);
   }
   return emax;
 }
 
 // Shared-memory state of one CTA of the tensor-core Kronecker kernels.
 struct TcState {
-  unsigned char* as;  // digit slices of the rows (7 x 4 KB)
-  unsigned char* bx;  // digit slices of the taps along x (7 x 512 B)
+  unsigned char* as;  // digit slices of the rows (kS x 4 KB)
+  unsigned char* bx;  // digit slices of the taps along x (kS x 512 B)
   unsigned char* by;  // along y
   double* V;          // the CTA's vectors, element (vi, x, y) at vi VP + y LP + x
   double* sc;         // diagonal of the slice, (x, y) at y LP + x
@@ -138,24 +220,26 @@ struct TcState {
   int* fail;          // a bounded wait gave up
   int ex, ey;         // exponents of the taps
   int Lx, Ly, LP, VP;
-  uint32_t tbase;     // TMEM accumulators (7 x 16 columns)
+  uint32_t tbase;     // TMEM accumulators (kS x 16 columns)
 };
 
 __host__ __device__ __forceinline__ int tc_pitch(int Lx) { return Lx | 1; }
 
+template <class Dg>
 __device__ __forceinline__ void tc_layout(TcState& s, unsigned char* sm, int nvpc, int Lx, int Ly) {
   s.as = sm;
-  s.bx = s.as + kS * kASlice;
-  s.by = s.bx + kS * kBSlice;
+  s.bx = s.as + Dg::kS * kASlice;
+  s.by = s.bx + Dg::kS * kBSlice;
   s.Lx = Lx;
   s.Ly = Ly;
   s.LP = tc_pitch(Lx);
   s.VP = Ly * s.LP;
-  s.V = reinterpret_cast<double*>(s.by + kS * kBSlice);
+  s.V = reinterpret_cast<double*>(s.by + Dg::kS * kBSlice);
   s.sc = s.V + nvpc * s.VP;
 }
 
 // TMEM, barrier and the digits of the taps of E_x, E_y (kind: E or E^{-1}).
+template <class Dg>
 __device__ void tc_setup(TcState& s, uint32_t* tmem_sh, const KronTaps& taps, bool inv, double* tx,
                          double* ty) {
   const int warp = threadIdx.x >> 5;
@@ -174,11 +258,11 @@ __device__ void tc_setup(TcState& s, uint32_t* tmem_sh, const KronTaps& taps, bo
     ty[threadIdx.x] = inv ? taps.eyi[threadIdx.x] : taps.ey[threadIdx.x];
   }
   // zero digits of k = 8 .. 15, which sides of at most 8 never write
-  for (int e = threadIdx.x; e < kS * kASlice / 16; e += blockDim.x)
+  for (int e = threadIdx.x; e < Dg::kS * kASlice / 16; e += blockDim.x)
     reinterpret_cast<uint4*>(s.as)[e] = make_uint4(0u, 0u, 0u, 0u);
   __syncthreads();
-  s.ex = tc_tap_digits(tx, s.Lx, s.bx);
-  s.ey = tc_tap_digits(ty, s.Ly, s.by);
+  s.ex = tc_tap_digits<Dg>(tx, s.Lx, s.bx);
+  s.ey = tc_tap_digits<Dg>(ty, s.Ly, s.by);
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
@@ -193,24 +277,13 @@ __device__ void tc_teardown(const TcState& s) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 128;" ::"r"(s.tbase));
 }
 
-// The number W 2^(e - 2102), W the integer sum of the accumulators, rounded to
-// FP64 (W's leading 53 bits; e: the sum of the two biased exponents).
-__device__ __forceinline__ double tc_compose(long long W, int e) {
-  const unsigned long long x = static_cast<unsigned long long>(W < 0 ? -W : W);
-  const int lz = __clzll(static_cast<long long>(x));
-  const unsigned long long m = ((x << (lz - 1)) + 0x200u) >> 10;  // 2^52 .. 2^53
-  const int ef = e - 1016 - lz;
-  if (x != 0 && (ef < 1 || ef > 2045)) return ldexp(static_cast<double>(W), e - 2102);
-  unsigned long long r = (static_cast<unsigned long long>(ef - 1) << 52) + m;
-  if (W < 0) r |= 0x8000000000000000ULL;
-  return (x == 0) ? 0.0 : __longlong_as_double(static_cast<long long>(r));
-}
-
 // One factor B on the nv vectors in s.V: the diagonal s.sc before the taps
 // (post = false: B, B^{-T}) or after them (post = true: B^T), then the x and
 // y steps as digit-sliced products.  All threads, which have synchronised since
 // s.V and s.sc were written; false if a wait gave up.
+template <class Dg>
 __device__ bool tc_slice(TcState& s, bool post, int nv, int& phase) {
+  constexpr int kS = Dg::kS;
   const int warp = threadIdx.x >> 5;
   const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((kK >> 3) << 17) | ((kR >> 4) << 24);
   const int r = threadIdx.x;  // the row of both products this thread owns
@@ -234,21 +307,21 @@ __device__ bool tc_slice(TcState& s, bool post, int nv, int& phase) {
           if (!post && dir == 0) x *= scp[k];
         }
         row[k] = x;
-        emax = max(emax, tc_exp(x));
+        emax = max(emax, Dg::expo(x));
       }
 #pragma unroll
       for (int half = 0; half < 2; ++half) {
         if (half == 1 && !wide) break;
         unsigned long long t[8];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) t[q] = tc_align(row[half * 8 + q], emax);
+        for (int q = 0; q < 8; ++q) t[q] = Dg::align(row[half * 8 + q], emax);
 #pragma unroll
         for (int p = 0; p < kS; ++p)
           *reinterpret_cast<uint4*>(s.as + p * kASlice + 2 * tc_off(r, half * 8)) =
-              make_uint4(tc_pack(tc_digit(t[0], p), tc_digit(t[1], p)),
-                         tc_pack(tc_digit(t[2], p), tc_digit(t[3], p)),
-                         tc_pack(tc_digit(t[4], p), tc_digit(t[5], p)),
-                         tc_pack(tc_digit(t[6], p), tc_digit(t[7], p)));
+              make_uint4(tc_pack(Dg::digit(t[0], p), Dg::digit(t[1], p)),
+                         tc_pack(Dg::digit(t[2], p), Dg::digit(t[3], p)),
+                         tc_pack(Dg::digit(t[4], p), Dg::digit(t[5], p)),
+                         tc_pack(Dg::digit(t[6], p), Dg::digit(t[7], p)));
       }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -276,10 +349,8 @@ __device__ bool tc_slice(TcState& s, bool post, int nv, int& phase) {
     const bool ok = __syncthreads_and(*s.fail == 0) != 0;
     asm volatile("tcgen05.fence::after_thread_sync;");
     if (!ok) return false;
-    // recombination, eight columns at a time: the accumulators are integers
-    // below 2^21, read off the low bits of 1.5 2^23 + P_d (as P_d + kM), and
-    // W = sum_d P_d 2^(44 - 8 d) (d = 6 rounded), below 2^63
-    const int e2 = emax + (dir == 0 ? s.ex : s.ey);
+    // recombination, eight columns at a time
+    const int eb = dir == 0 ? s.ex : s.ey;
 #pragma unroll
     for (int half = 0; half < 2; ++half) {
       if (half * 8 >= klen) break;
@@ -299,17 +370,10 @@ __device__ bool tc_slice(TcState& s, bool post, int nv, int& phase) {
         for (int jq = 0; jq < 8; ++jq) {
           const int j = half * 8 + jq;
           if (j >= klen) continue;
-          constexpr uint32_t kM = 0x4B400000u;
-          uint32_t u[kS];
+          uint32_t pd[kS];
 #pragma unroll
-          for (int d = 0; d < kS; ++d) u[d] = __float_as_uint(__uint_as_float(acc[d][jq]) + 12582912.0f);
-          const int a = static_cast<int>(u[0] * 256u + u[1] - kM * 257u);
-          const int b = static_cast<int>(u[2] * 256u + u[3] - kM * 257u);
-          const int c = static_cast<int>(u[4] * 256u + u[5] - kM * 257u);
-          const int g = static_cast<int>(u[6] - kM);
-          const long long W = ((static_cast<long long>(a) * 65536 + b) << 20) +
-                              (static_cast<long long>(c) << 4) + ((g + 8) >> 4);
-          double val = tc_compose(W, e2);
+          for (int d = 0; d < kS; ++d) pd[d] = acc[d][jq];
+          double val = Dg::compose(pd, emax, eb);
           // rows are read above and written only here, each by its owner
           if (post && dir == 1) val *= scp[j * step];
           v[j * step] = val;
@@ -326,6 +390,7 @@ __device__ bool tc_slice(TcState& s, bool post, int nv, int& phase) {
 
 // One CTA per (group of nvpc vectors, batch entry); the arguments and slice
 // ranges are those of k_kron_rows<double>.
+template <class Dg>
 __global__ void __launch_bounds__(kTC) k_kron_tc(const double* in, double* out, KronArgs a,
                                                 int nvpc, int* status) {
   const int b = blockIdx.y;
@@ -349,7 +414,7 @@ __global__ void __launch_bounds__(kTC) k_kron_tc(const double* in, double* out, 
   __shared__ int fail_sh;
   __shared__ double tx[kMaxSide], ty[kMaxSide];
   TcState s;
-  tc_layout(s, tc_sm, nvpc, a.Lx, a.Ly);
+  tc_layout<Dg>(s, tc_sm, nvpc, a.Lx, a.Ly);
   s.mbar = &mbar;
   s.fail = &fail_sh;
   const double* src = in + static_cast<size_t>(b) * a.mat_stride;
@@ -359,7 +424,7 @@ __global__ void __launch_bounds__(kTC) k_kron_tc(const double* in, double* out, 
     if (a.vscale) val *= a.vscale[static_cast<size_t>(b) * a.vscale_stride + v0 + vi];
     s.V[vi * s.VP + y * s.LP + i - y * a.Lx] = val;
   }
-  tc_setup(s, &tmem_sh, a.taps, a.kind == kBIT, tx, ty);
+  tc_setup<Dg>(s, &tmem_sh, a.taps, a.kind == kBIT, tx, ty);
   const double up = (a.kind == kBIT) ? a.emc : a.ec, dn = (a.kind == kBIT) ? a.ec : a.emc;
   const int8_t* f = a.field + static_cast<size_t>(chain) * a.L * N;
   int phase = 0;
@@ -371,7 +436,7 @@ __global__ void __launch_bounds__(kTC) k_kron_tc(const double* in, double* out, 
       s.sc[y * s.LP + i - y * a.Lx] = f[static_cast<size_t>(l0) * N + i] > 0 ? up : dn;
     }
     __syncthreads();
-    ok = tc_slice(s, a.kind == kBT, nv, phase);
+    ok = tc_slice<Dg>(s, a.kind == kBT, nv, phase);
   }
   if (!ok && threadIdx.x == 0) atomicExch(status, kDevTimeout);
   __syncthreads();
@@ -389,6 +454,7 @@ __global__ void __launch_bounds__(kTC) k_kron_tc(const double* in, double* out, 
 // element is added to the bin of its separation (spin-up G(l,0) bins or Y
 // bins of slice l): one thread per bin sums its element of each of the CTA's
 // vectors and adds the sum to bins[chain][l][slot].
+template <class Dg>
 __global__ void __launch_bounds__(kTC) k_gtau_tc(const double* Xall, GtauArgs a, int nvpc,
                                                 int* status) {
   const int b = blockIdx.y;
@@ -403,7 +469,7 @@ __global__ void __launch_bounds__(kTC) k_gtau_tc(const double* Xall, GtauArgs a,
   __shared__ int fail_sh;
   __shared__ double tx[kMaxSide], ty[kMaxSide];
   TcState s;
-  tc_layout(s, tc_sm, nvpc, a.Lx, a.Ly);
+  tc_layout<Dg>(s, tc_sm, nvpc, a.Lx, a.Ly);
   s.mbar = &mbar;
   s.fail = &fail_sh;
   const double* X = Xall + static_cast<size_t>(b) * a.mat_stride;
@@ -411,7 +477,7 @@ __global__ void __launch_bounds__(kTC) k_gtau_tc(const double* Xall, GtauArgs a,
     const int vi = e / N, i = e - vi * N, y = i / a.Lx;
     s.V[vi * s.VP + y * s.LP + i - y * a.Lx] = X[static_cast<size_t>(v0) * N + e];
   }
-  tc_setup(s, &tmem_sh, a.taps, a.kind == kBIT, tx, ty);
+  tc_setup<Dg>(s, &tmem_sh, a.taps, a.kind == kBIT, tx, ty);
   const int8_t* f = a.field + static_cast<size_t>(chain) * a.L * N;
   const double up = (a.kind == kBIT) ? a.emc : a.ec, dn = (a.kind == kBIT) ? a.ec : a.emc;
   int phase = 0;
@@ -423,7 +489,7 @@ __global__ void __launch_bounds__(kTC) k_gtau_tc(const double* Xall, GtauArgs a,
         s.sc[y * s.LP + i - y * a.Lx] = f[static_cast<size_t>(l - 1) * N + i] > 0 ? up : dn;
       }
       __syncthreads();
-      ok = tc_slice(s, false, nv, phase);
+      ok = tc_slice<Dg>(s, false, nv, phase);
       if (!ok) break;
     }
     double* out = a.bins + ((static_cast<size_t>(chain) * (a.L + 1) + l) * 2 + a.bin_slot) * N;
@@ -454,35 +520,50 @@ __global__ void __launch_bounds__(kTC) k_gtau_tc(const double* Xall, GtauArgs a,
 
 int kron_tc_vectors(int Lx, int Ly) { return kR / max(Lx, Ly); }
 
+template <class Dg>
 static size_t tc_bytes(int nvpc, int Lx, int Ly) {
-  return static_cast<size_t>(kS) * kASlice + 2ull * kS * kBSlice +
+  return static_cast<size_t>(Dg::kS) * kASlice + 2ull * Dg::kS * kBSlice +
          static_cast<size_t>(nvpc + 1) * Ly * tc_pitch(Lx) * sizeof(double);
+}
+
+template <class Dg>
+static cudaError_t tc_launch_kron(const double* in, double* out, int batch, const KronArgs& a,
+                                  int* status, cudaStream_t st) {
+  const int nvpc = kron_tc_vectors(a.Lx, a.Ly);
+  const size_t smem = tc_bytes<Dg>(nvpc, a.Lx, a.Ly);
+  cudaError_t e = cudaFuncSetAttribute(k_kron_tc<Dg>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       static_cast<int>(smem));
+  if (e != cudaSuccess) return e;
+  dim3 grid((a.N + nvpc - 1) / nvpc, batch);
+  k_kron_tc<Dg><<<grid, kTC, smem, st>>>(in, out, a, nvpc, status);
+  return cudaGetLastError();
+}
+
+template <class Dg>
+static cudaError_t tc_launch_gtau(const double* X, int batch, const GtauArgs& a, int* status,
+                                  cudaStream_t st) {
+  const int nvpc = kron_tc_vectors(a.Lx, a.Ly);
+  const size_t smem = tc_bytes<Dg>(nvpc, a.Lx, a.Ly);
+  cudaError_t e = cudaFuncSetAttribute(k_gtau_tc<Dg>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       static_cast<int>(smem));
+  if (e != cudaSuccess) return e;
+  dim3 grid((a.N + nvpc - 1) / nvpc, batch);
+  k_gtau_tc<Dg><<<grid, kTC, smem, st>>>(X, a, nvpc, status);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_kron_tc(const double* in, double* out, int batch, const KronArgs& a, int* status,
                            cudaStream_t st) {
   if (a.Lx > kK || a.Ly > kK) return cudaErrorInvalidValue;
-  const int nvpc = kron_tc_vectors(a.Lx, a.Ly);
-  const size_t smem = tc_bytes(nvpc, a.Lx, a.Ly);
-  cudaError_t e = cudaFuncSetAttribute(k_kron_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
-  if (e != cudaSuccess) return e;
-  dim3 grid((a.N + nvpc - 1) / nvpc, batch);
-  k_kron_tc<<<grid, kTC, smem, st>>>(in, out, a, nvpc, status);
-  return cudaGetLastError();
+  return a.digits8 ? tc_launch_kron<TcDigits8>(in, out, batch, a, status, st)
+                   : tc_launch_kron<TcDigits7>(in, out, batch, a, status, st);
 }
 
 cudaError_t launch_gtau_tc(const double* X, int batch, const GtauArgs& a, int* status,
                            cudaStream_t st) {
   if (a.Lx > kK || a.Ly > kK) return cudaErrorInvalidValue;
-  const int nvpc = kron_tc_vectors(a.Lx, a.Ly);
-  const size_t smem = tc_bytes(nvpc, a.Lx, a.Ly);
-  cudaError_t e = cudaFuncSetAttribute(k_gtau_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
-  if (e != cudaSuccess) return e;
-  dim3 grid((a.N + nvpc - 1) / nvpc, batch);
-  k_gtau_tc<<<grid, kTC, smem, st>>>(X, a, nvpc, status);
-  return cudaGetLastError();
+  return a.digits8 ? tc_launch_gtau<TcDigits8>(X, batch, a, status, st)
+                   : tc_launch_gtau<TcDigits7>(X, batch, a, status, st);
 }
 
 }  // namespace dqmc

@@ -50,47 +50,7 @@ namespace {
 
 namespace cg = cooperative_groups;
 
-constexpr int kNB = 32;  // panel width
-
-// log2 of the squared norm of x[0 .. len) as an FP32 sort key, from the
-// exponent fields and the FP32 mantissas (the order only steers the
-// numerics; any order gives an exact factorisation).  One warp, len <= kMaxN;
-// every element is loaded once, all loads of a lane in flight together.  The
-// key is returned on every lane: +3e38 for Inf/NaN entries, -3e38 for a zero
-// vector.
-__device__ __forceinline__ float qb_norm_key(const double* x, int len, int lane) {
-  constexpr int kR = kMaxN / 32;
-  long long bits[kR];
-#pragma unroll
-  for (int t = 0; t < kR; ++t) {
-    const int r = lane + 32 * t;
-    bits[t] = (r < len) ? __double_as_longlong(x[r]) : 0LL;
-  }
-  int emax = 0;
-  bool bad = false;
-#pragma unroll
-  for (int t = 0; t < kR; ++t) {
-    const int E = static_cast<int>((bits[t] >> 52) & 0x7FF);
-    bad |= (E == 0x7FF);
-    emax = max(emax, E);
-  }
-  for (int o = 16; o > 0; o >>= 1) emax = max(emax, __shfl_xor_sync(0xFFFFFFFFu, emax, o));
-  bad = __any_sync(0xFFFFFFFFu, bad);
-  float s = 0.0f;
-#pragma unroll
-  for (int t = 0; t < kR; ++t) {
-    const int E = static_cast<int>((bits[t] >> 52) & 0x7FF);
-    if (E != 0) {
-      const float mt = __int_as_float(0x3F800000 | static_cast<int>((bits[t] >> 29) & 0x7FFFFF));
-      const float y = ldexpf(mt, E - emax);
-      s = fmaf(y, y, s);
-    }
-  }
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
-  if (bad) return 3.0e38f;
-  if (emax == 0) return -3.0e38f;
-  return 2.0f * static_cast<float>(emax - 1023) + __log2f(s);
-}
+constexpr int kNB = kQrbNB;
 
 constexpr int kPCS = 4;             // CTAs per matrix (one cluster)
 constexpr int kPCW = kNB / kPCS;    // column warps per CTA
@@ -550,7 +510,8 @@ static size_t qb_panel_smem(int w, int m) {
 
 cudaError_t launch_qr_blocked(double* Xt, long long sX, double* Qt, long long sQ, double* D,
                               long long sD, double* Rtil, long long sR, const QrbWork& wk, int n,
-                              int batch, void* oz, int oz_batch, int* status, cudaStream_t st) {
+                              int batch, void* oz, int oz_batch, int* status, cudaStream_t st,
+                              bool split_rows) {
   if (n <= 0 || batch <= 0 || n > kMaxN) return n > kMaxN ? cudaErrorInvalidValue : cudaSuccess;
   double* WA = wk.W0;
   double* WB = wk.W1;
@@ -567,7 +528,10 @@ cudaError_t launch_qr_blocked(double* Xt, long long sX, double* Qt, long long sQ
     const double* src = (p == 0) ? Xt : ((p & 1) ? WA : WB);
     const long long sSrc = (p == 0) ? sX : sW;
     double* dst = (p & 1) ? WB : WA;
-    {  // one cluster per matrix
+    if (split_rows) {
+      e = launch_qr_panel2(src, sSrc, dst, sW, wk.perm, Vt, sR, Yt, sX, D, sD, n, c0, w, batch,
+                           status, st);
+    } else {  // one cluster per matrix
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(kPCS * batch, 1, 1);
       cfg.blockDim = dim3(kPT, 1, 1);

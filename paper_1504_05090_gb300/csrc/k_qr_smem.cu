@@ -458,11 +458,12 @@ cudaError_t qs_launch(double* Xt, long long sX, double* Qt, long long sQ, double
 }  // namespace
 
 // CTAs per matrix of k_qr_smem, or 0 where another kernel takes the matrix.
-// The choice of kernel depends on n alone, so that a chain's numbers do not
-// depend on how many chains share its context (the result does not depend on
-// the CTAs either).  Measured (us for the batch, GB300): this kernel against
-// the blocked QR (the default mode's alternative from n = 64 on) and the
-// column-pivoted QR on global memory (k_qrp_cluster):
+// The choice of kernel depends on n and the group's interval alone (stack_qr in
+// dqmc.cu), so that a chain's numbers do not depend on how many chains share its
+// context (the result does not depend on the CTAs either).  Measured (us for the
+// batch, GB300): this kernel against the blocked QR (the default mode's
+// alternative from n = 64 on) and the column-pivoted QR on global memory
+// (k_qrp_cluster):
 //   n = 16:  32 matrices 45 / - / 124; 256: 46 / - / 463
 //   n = 36:  32: 106 / - / 278;       256: 127 / - / 1083
 //   n = 64:  32: 258 / 580 / 531;     256: 353 / 1987 / 2076; 1024: 1257 / 6884 / 7369

@@ -41,6 +41,7 @@ struct KronArgs {
   // if it is < cp[blk+1] (0-based slice index), else leaves the matrix as is.
   const int* cp;
   int step;
+  int digits8;           // launch_kron_tc: eight 7-bit digits instead of seven of 8 bits
 };
 
 // Batched square FP64 GEMM with diagonal scalings:
@@ -157,7 +158,9 @@ cudaError_t launch_qr_smem(int cs, double* Xt, long long sX, double* Qt, long lo
 // it, and the trailing updates and the accumulation of Q run on the
 // tensor-core products (oz: scratch of ozaki_scratch_bytes(n, oz_batch)).
 // X and Rtil double as workspace; QrbWork adds two n x n buffers W0, W1, Wt
-// (n x 32) and perm (n ints) per matrix.
+// (n x 32) and perm (n ints) per matrix.  split_rows: the panels are formed by
+// two CTAs with the rows split between them (k_qr_panel2.cu) instead of four
+// with the columns split.
 struct QrbWork {
   double* W0; double* W1; long long sW;
   double* Wt; long long sWt;
@@ -165,7 +168,14 @@ struct QrbWork {
 };
 cudaError_t launch_qr_blocked(double* Xt, long long sX, double* Qt, long long sQ, double* D,
                               long long sD, double* Rtil, long long sR, const QrbWork& wk, int n,
-                              int batch, void* oz, int oz_batch, int* status, cudaStream_t st);
+                              int batch, void* oz, int oz_batch, int* status, cudaStream_t st,
+                              bool split_rows);
+// One panel of it, columns c0 .. c0 + w - 1 (the arguments of k_qrb_panel).
+constexpr int kQrbNB = 32;  // panel width
+cudaError_t launch_qr_panel2(const double* Ws, long long sWs, double* Wd, long long sWd, int* perm,
+                             double* Vt, long long sV, double* Yt, long long sY, double* D,
+                             long long sD, int n, int c0, int w, int batch, int* status,
+                             cudaStream_t st);
 // Kernel launches of one launch_qr_blocked call.
 int qr_blocked_launches(int n, int batch, int oz_batch);
 // Gauss-Jordan: A (overwritten) -> Ainv, out of place; logabs may be null.
@@ -197,6 +207,7 @@ struct GtauArgs {
   long long mat_stride;
   double* bins;          // [chain][L+1][2][N]
   int bin_slot;          // 0 for G(l,0), 1 for Y
+  int digits8;           // launch_gtau_tc: as KronArgs
 };
 // pair: propagate in float pairs (groups whose working precision is df32).
 cudaError_t launch_gtau_propagate(double* X, int batch, const GtauArgs& a, bool pair,
