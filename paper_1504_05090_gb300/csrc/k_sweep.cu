@@ -529,11 +529,14 @@ __global__ void __launch_bounds__(kMetroThreads + (kScalarWarp<T>() ? 32 : 0)) k
   };
   auto row_entry = [&](int i) -> Entry {  // the own entries of row i
     if constexpr (kBoth) {
-      if (i >= rq) return ld_row(i);  // further ahead than the ring
+      // a slot is asked for again only once its copy has landed (groups are not
+      // ordered against each other): the rows up to i are those of the groups
+      // waited for here
       if (i >= pbase)
         asm volatile("cp.async.wait_group 0;" ::: "memory");
       else
         asm volatile("cp.async.wait_group 1;" ::: "memory");
+      if (i >= rq) return ld_row(i);  // further ahead than the ring
       Entry e;
       e.x[0] = ring[(i % kRing) * NP + cj];
       return e;
@@ -750,7 +753,8 @@ __global__ void __launch_bounds__(kMetroThreads + (kScalarWarp<T>() ? 32 : 0)) k
         flush_sh[1] = (i < N) ? i : -1;
       }
     }
-    // flush, by all warps
+    // flush, by all warps; no copy of a row may be under way while G is rewritten
+    if constexpr (kBoth) asm volatile("cp.async.wait_group 0;" ::: "memory");
     if (cs > 1)
       peer_barrier<true>(xbar, cs, rank, xphase, a.status, &xbroken);
     else
