@@ -28,6 +28,13 @@ __device__ __forceinline__ double scale_of(const double* p, int mode, int i) {
   }
 }
 
+// rs acc cs + beta C, each rounding written out: left to the compiler, the two
+// GEMM kernels contract the expression differently and differ in the last bit.
+__device__ __forceinline__ double gemm_out(double beta, double rs, double acc, double cs, const double* C) {
+  const double t = __dmul_rn(rs, acc);
+  return (beta != 0.0) ? __fma_rn(t, cs, __dmul_rn(beta, *C)) : __dmul_rn(t, cs);
+}
+
 // ---------------------------------------------------------------------------
 // Batched FP64 GEMM, 64x64 output tile per CTA, 16x16 threads with 4x4 each.
 // ---------------------------------------------------------------------------
@@ -106,10 +113,8 @@ __global__ void __launch_bounds__(256) k_gemm_f64(GemmArgs a) {
     for (int q = 0; q < 4; ++q) {
       const int j = j0 + tx * 4 + q;
       if (j >= n) continue;
-      double v = rv * acc[r][q] * csv[tx * 4 + q];
       const size_t o = static_cast<size_t>(i) * n + j;
-      if (a.beta != 0.0) v += a.beta * C[o];
-      C[o] = v;
+      C[o] = gemm_out(a.beta, rv, acc[r][q], csv[tx * 4 + q], C + o);
     }
   }
 }
@@ -135,7 +140,7 @@ __global__ void __launch_bounds__(kGsThreads) k_gemm_small(GemmArgs a, int R) {
   double* Bs = gs_mem;         // [n][ldb]
   double* As = Bs + n * ldb;   // [R][n]
   __shared__ double rsv[64], csv[64], ksv[64];
-  {  // scale factors: a third of the warps each for rows, columns, inner index
+  {  // scale factors of the rows, the columns and the inner index
     const double* rs = a.rs ? a.rs + b * a.srs : nullptr;
     const double* ks = a.ks ? a.ks + b * a.sks : nullptr;
     const double* cs = a.cs ? a.cs + b * a.scs : nullptr;
@@ -175,10 +180,8 @@ __global__ void __launch_bounds__(kGsThreads) k_gemm_small(GemmArgs a, int R) {
     double acc = 0.0;
 #pragma unroll 4
     for (int k = 0; k < n; ++k) acc = fma(ar[k], bc[k * ldb], acc);
-    double v = rsv[i] * acc * csv[j];
     const size_t o = static_cast<size_t>(i0 + i) * n + j;
-    if (a.beta != 0.0) v += a.beta * C[o];
-    C[o] = v;
+    C[o] = gemm_out(a.beta, rsv[i], acc, csv[j], C + o);
   }
 }
 

@@ -19,7 +19,8 @@ pytestmark = pytest.mark.gpu
 GOLDEN = os.path.join(os.path.dirname(os.path.abspath(__file__)), "golden", "gtau_long_step.npz")
 
 
-@pytest.mark.parametrize("Lx,Ly,prec,beta", [(8, 8, "df32", 20.0), (12, 12, "fp64", 8.0), (14, 14, "df32", 8.0)])
+@pytest.mark.parametrize("Lx,Ly,prec,beta", [(6, 6, "df32", 20.0), (10, 6, "fp64", 20.0), (8, 8, "df32", 20.0),
+                                             (12, 12, "fp64", 8.0), (14, 14, "df32", 8.0)])
 def test_gtau_is_reproduced(Lx, Ly, prec, beta):
     import paper_1504_05090_gb300 as pkg
     g = pkg.Group(Lx=Lx, Ly=Ly, t=0.25, U=2.0, beta=beta, dtau=0.4, n_chains=2, stab_interval=8,
