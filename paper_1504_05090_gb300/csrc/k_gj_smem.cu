@@ -29,6 +29,7 @@
 #include <cfloat>
 
 #include "common.cuh"
+#include "gj_key.cuh"
 #include "kernels.h"
 
 namespace cg = cooperative_groups;
@@ -50,14 +51,20 @@ size_t gs_smem(int n, int cs) {
   return (static_cast<size_t>((n + cs - 1) / cs) * ld + ld + (cs > 1 ? 2 * cs * ld : 0)) * 8;
 }
 
-// Pivot keys: the bits of |x| (its high word for FP64) order as the numbers.
+// Pivot keys: the bits of |x| (rounded to FP32 for FP64, as k_gj_cluster
+// compares it) order as the numbers.
 __device__ __forceinline__ unsigned gs_key(double x) {
-  return static_cast<unsigned>(__double2hiint(x)) & 0x7FFFFFFFu;
+  bool ok;
+  const unsigned k = gj_key_bits(static_cast<uint64_t>(__double_as_longlong(x)), ok);
+  return ok ? k : static_cast<unsigned>(__float_as_int(static_cast<float>(absd(x))));
 }
 __device__ __forceinline__ unsigned gs_key(df32 x) {
   return static_cast<unsigned>(__float_as_int(x.hi)) & 0x7FFFFFFFu;
 }
-__device__ __forceinline__ bool gs_bad(double, unsigned key) { return key >= 0x7FF00000u; }
+// Inf or NaN as the pivot (FP64: finite numbers beyond FP32's range are not)
+__device__ __forceinline__ bool gs_bad(double piv, unsigned) {
+  return (static_cast<unsigned>(__double2hiint(piv)) & 0x7FFFFFFFu) >= 0x7FF00000u;
+}
 __device__ __forceinline__ bool gs_bad(df32, unsigned key) { return key >= 0x7F800000u; }
 __device__ __forceinline__ double gs_d(double x) { return x; }
 __device__ __forceinline__ double gs_d(df32 x) { return static_cast<double>(x); }
@@ -202,7 +209,7 @@ __global__ void __launch_bounds__(kGT) k_gj_smem(const double* Aall, long long s
       ip[pg] = static_cast<short>(k);
       pivs[k] = c.piv;
       if (p >= 0) used[p] = 1;
-      if (gs_bad(inv, c.key)) atomicExch(status, kDevNonFinite);
+      if (gs_bad(T(c.piv), c.key)) atomicExch(status, kDevNonFinite);
       if (c.key == 0u && (__double_as_longlong(c.piv) << 1) == 0LL) atomicExch(status, kDevSingular);
     }
     __syncthreads();
