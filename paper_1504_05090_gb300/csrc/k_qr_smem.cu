@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(kQT, 2) k_qr_smem(double* Xall, long long sX, 
   __shared__ unsigned char live[2][kMaxN / CS], rec[kMaxN / CS], colof[kMaxN / CS == kMaxN ? kMaxN : 1];
   __shared__ short stepof[kMaxN / CS];
   __shared__ Cand cand[2][CS];  // by step parity and CTA
-  __shared__ int wait_sum[2];
+  __shared__ int wait_sum[2], stale[2];
   __shared__ double kap_sh, vj_sh;
   __shared__ double vjs[CS == 1 ? kMaxN : 1];  // v_j[j]
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -127,7 +127,10 @@ __global__ void __launch_bounds__(kQT, 2) k_qr_smem(double* Xall, long long sX, 
     live[0][i] = static_cast<unsigned char>(i);
     stepof[i] = static_cast<short>(n);
   }
-  if (tid < 2) wait_sum[tid] = 0;
+  if (tid < 2) {
+    wait_sum[tid] = 0;
+    stale[tid] = -1;
+  }
   __syncthreads();
   for (int g = w; 8 * g < ncol; g += nw) {
     const int c = 8 * g + lg;
@@ -244,6 +247,19 @@ __global__ void __launch_bounds__(kQT, 2) k_qr_smem(double* Xall, long long sX, 
         a = qs_lsum<4>(a);
         if (l4 == 0 && i < m) dsum[c] = a;
       }
+      if constexpr (CS > 1) {
+        // the sum that the own candidate missed (below), if it lost
+        const int c = stale[j & 1];
+        if (c >= 0 && c != lp && wu == ((m + 7) >> 3) % nu) {
+          const double* x = Xs + c * ld + l4;
+          const int t1 = j >> 2;
+          double a = (4 * t1 + l4 >= j) ? x[4 * t1] * x[4 * t1] : 0.0;
+#pragma unroll 4
+          for (int t = t1 + 1; t < nslots; ++t) a = fma(x[4 * t], x[4 * t], a);
+          a = qs_lsum<4>(a);
+          if (lane == 0) n1[c] = n2[c] = a;
+        }
+      }
     }
     __syncthreads();
     // 2. factors of the live columns
@@ -273,6 +289,10 @@ __global__ void __launch_bounds__(kQT, 2) k_qr_smem(double* Xall, long long sX, 
     const int np = ahead ? best(lv, m, lp) : -1;
     if (ahead && w == ws) {
       if (j + 1 < n) prepare(j + 1, np, xp, true);
+      // a candidate that loses to another CTA's stays live and needs its norm
+      // summed afresh like the other columns (as with CS = 1); the next step
+      // does so beside its dot products
+      if (CS > 1 && lane == 0) stale[(j + 1) & 1] = (np >= 0 && rec[np]) ? np : -1;
     } else if (!ahead || helper) {
       const int wi = ahead ? wu : w, wn = ahead ? nu : nw;
       for (int g = wi; 8 * g < m; g += wn) {
@@ -329,8 +349,10 @@ __global__ void __launch_bounds__(kQT, 2) k_qr_smem(double* Xall, long long sX, 
     }
     if (!ahead) {
       __syncthreads();
-      if (w == ws && j + 1 < n)
+      if (w == ws && j + 1 < n) {
         prepare(j + 1, best(lv, m, lp), nullptr, false);
+        if (CS > 1 && lane == 0) stale[(j + 1) & 1] = -1;
+      }
     }
     m = ml;
   }

@@ -46,3 +46,38 @@ def test_result_does_not_depend_on_the_ctas_per_matrix(Lx, Ly, counts):
         if first is None:
             first = got
         assert np.array_equal(got[0], first[0]) and np.array_equal(got[1], first[1])
+
+
+def _layered(rng, count, L, Lx, Ly):
+    """Staggered fields with a random sign per slice and fields of a random sign
+    per row times one per column: many columns whose norms tie or nearly do."""
+    x, y = np.meshgrid(np.arange(Lx), np.arange(Ly))
+    out = np.empty((count, L, Ly, Lx), dtype=np.int8)
+    for c in range(count):
+        if c & 1:
+            out[c] = rng.choice([-1, 1], size=(Ly, 1)) * rng.choice([-1, 1], size=(1, Lx))
+        else:
+            out[c] = rng.choice([-1, 1], size=(L, 1, 1)) * np.where((x + y) % 2, 1, -1)
+    return out.reshape(count, L, Lx * Ly)
+
+
+@pytest.mark.parametrize("Lx,Ly,counts", [(10, 8, (40,)), (10, 10, (40,)), (12, 12, (40, 10))])
+def test_pivots_of_graded_symmetric_fields_do_not_depend_on_the_ctas(Lx, Ly, counts):
+    """U = 8: columns lose most of their norm in a step, so that norms are summed
+    afresh all the time; every chain, bit for bit, against one CTA per matrix."""
+    import paper_1504_05090_gb300 as pkg
+
+    def grp(C):
+        return _grp(Lx, Ly, C=C, U=8.0, beta=10.0, dtau=0.25, ns=4)
+
+    f = _layered(np.random.default_rng(0), 240, 40, Lx, Ly)
+    for b0 in range(0, len(f), 80):
+        with pkg.DQMC([grp(80)], seed=0) as sim:
+            sim.set_field([f[b0:b0 + 80]])
+            ref = [sim.G(c, 0) for c in range(80)]
+        for C in counts:
+            with pkg.DQMC([grp(C)], seed=0) as sim:
+                for q in range(0, 80, C):
+                    sim.set_field([f[b0 + q:b0 + q + C]])
+                    for c in range(C):
+                        assert np.array_equal(sim.G(c, 0), ref[q + c]), (b0, q, c, C)
