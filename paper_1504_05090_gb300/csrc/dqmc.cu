@@ -350,7 +350,7 @@ GemmArgs gemm0(int n) {
 // N >= kOzakiMinN unless the context asks for the FP64 pipe.
 cudaError_t gemm(dqmc_ctx* ctx, Group& g, const GemmArgs& m, int batch) {
   if (ctx->gemm_mode == DQMC_GEMM_TENSOR && g.oz) {
-    ctx->launches += gemm_ozaki_launches(m, batch, g.oz_batch) - 1;
+    ctx->launches += ozaki_product_launches(m.n, m.n, m.n, m.balance != 0, batch, g.oz_batch) - 1;
     return launch_gemm_ozaki(m, batch, g.oz, g.oz_batch, ctx->d_status, g.st);
   }
   return launch_gemm(m, batch, g.st);
@@ -467,6 +467,7 @@ cudaError_t invert(dqmc_ctx* ctx, Group& g, double* A, double* Ainv, int batch, 
   const int cs = gj_smem_ctas(g.N, conc, ctx->nsm, pair);
   if (cs > 0)
     return launch_gj_smem(cs, A, g.nn(), Ainv, g.nn(), g.N, batch, logabs, ctx->d_status, g.st, pair);
+  if (pair) ++ctx->launches;  // A into float pairs first
   return launch_gj_cluster(A, g.nn(), Ainv, g.nn(), g.N, batch, logabs, ctx->d_status, g.st, pair);
 }
 

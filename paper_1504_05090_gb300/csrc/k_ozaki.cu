@@ -1399,10 +1399,12 @@ cudaError_t launch_ozaki_product(const OzProduct& g, int batch, void* scratch, i
   return oz_run<64>(g, batch, scratch, max_batch, status, st);
 }
 
-int gemm_ozaki_launches(const GemmArgs& g, int batch, int max_batch) {
-  if (g.n <= kQN) return 1;
-  // the split and the product (plus the balance pass) per chunk of the batch
-  return (batch + max_batch - 1) / max_batch * (g.balance ? 3 : 2);
+int ozaki_product_launches(int M, int Nc, int K, bool balance, int batch, int max_batch) {
+  if (M <= kQN && Nc <= kQN && K <= kQN) return 1;
+  // the product, after its split if that is a kernel of its own and the balance
+  // pass, per chunk of the batch
+  const int per = (K <= 64 || Nc <= 32) ? 1 : 2;
+  return (batch + max_batch - 1) / max_batch * (per + (balance ? 1 : 0));
 }
 
 cudaError_t launch_gemm_ozaki(const GemmArgs& g, int batch, void* scratch, int max_batch,

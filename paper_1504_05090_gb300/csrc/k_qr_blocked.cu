@@ -495,12 +495,16 @@ OzProduct qb_prod(int M, int Nc, int K, const double* A, long long sA, long long
 }  // namespace
 
 int qr_blocked_launches(int n, int batch, int oz_batch) {
-  const int panels = (n + kNB - 1) / kNB;
-  const int chunks = (batch + oz_batch - 1) / oz_batch;
-  // identity and finalize; one panel kernel per panel; two products (one
-  // kernel per chunk of the batch) per panel except the last, which has no
-  // trailing columns, and two per panel of the Q accumulation
-  return 2 + panels + (4 * panels - 2) * chunks;
+  int sum = 2;  // identity and finalize
+  for (int c0 = 0; c0 < n; c0 += kNB) {
+    const int w = std::min(kNB, n - c0), m = n - c0, nt = m - w;
+    auto products = [&](int M, int Nc, int K) {
+      return ozaki_product_launches(M, Nc, K, false, batch, oz_batch);
+    };
+    // the panel; its trailing columns, of which the last one has none; Q
+    sum += 1 + (nt > 0 ? products(nt, w, m) + products(nt, m, w) : 0) + products(m, w, m) + products(m, m, w);
+  }
+  return sum;
 }
 
 // Dynamic shared memory of a panel of w columns, m rows.

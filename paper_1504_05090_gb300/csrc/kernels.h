@@ -112,8 +112,9 @@ cudaError_t launch_gemm(const GemmArgs& a, int batch, cudaStream_t st);
 size_t ozaki_scratch_bytes(int n, int max_batch);
 cudaError_t launch_gemm_ozaki(const GemmArgs& a, int batch, void* scratch, int max_batch,
                               int* status, cudaStream_t st);
-// Kernel launches of one launch_gemm_ozaki call.
-int gemm_ozaki_launches(const GemmArgs& a, int batch, int max_batch);
+// Kernel launches of one launch_ozaki_product call (launch_gemm_ozaki: M = Nc =
+// K = n).
+int ozaki_product_launches(int M, int Nc, int K, bool balance, int batch, int max_batch);
 // General form of the same tensor-core product: for each batch entry b,
 //   C[i*ldc + j] = alpha rs_i sum_k opA(i,k) ks_k opB(k,j) cs_j + beta C[i*ldc + j]
 // with opA(i,k) = A[i a_sv + k a_sk] (i < M, k < K) and opB(k,j) = B[j b_sv + k b_sk]
