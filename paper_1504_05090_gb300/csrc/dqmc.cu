@@ -101,7 +101,6 @@ struct Group {
   double *logabs = nullptr, *obs = nullptr, *drift = nullptr, *bins = nullptr, *gacc = nullptr;
   double* spin = nullptr;  // [C][N] accumulated spin correlation C(r)
   double* gout = nullptr;  // [C][L+1][N] staging of G(tau) for host output
-  double* qrs = nullptr;   // [C][2N] column norms of the QR
   void* oz = nullptr;      // digit slices of the tensor-core FP64 GEMM
   int oz_batch = 0;
   QrbWork qrb{};           // blocked-QR workspace (tensor-core path)
@@ -356,15 +355,21 @@ cudaError_t gemm(dqmc_ctx* ctx, Group& g, const GemmArgs& m, int batch) {
   return launch_gemm(m, batch, g.st);
 }
 
+// CTAs per matrix of the QR in shared memory, 0 where the group's stacks are
+// left to the others.
+int qr_ctas(const dqmc_ctx* ctx, const Group& g) {
+  return g.long_step ? 0 : qr_smem_ctas(g.N, ctx->total, ctx->nsm);
+}
+
 // QR of the stack step X = B..B (U D) (rows of g.X = columns of X) into the
 // stack entry (Q^T at Qt, D at Dv) and g.Rtil: column-pivoted with the matrix
-// in shared memory up to N = 144 (qr_smem_ctas; not where a step stretches far,
+// in shared memory up to N = 144 (qr_ctas; not where a step stretches far,
 // see kLongStep), else the blocked QR with tensor-core updates where the
 // tensor-core products are in use, else the column-pivoted cluster QR on global
 // memory.
 cudaError_t stack_qr(dqmc_ctx* ctx, Group& g, double* Qt, double* Dv) {
   const long long sD = static_cast<long long>(g.nc + 1) * g.N;
-  const int cs = g.long_step ? 0 : qr_smem_ctas(g.N, ctx->total, ctx->nsm);
+  const int cs = qr_ctas(ctx, g);
   if (cs > 0)
     return launch_qr_smem(cs, g.X, g.nn(), Qt, g.sstride(), Dv, sD, g.Rtil, g.nn(), g.N, g.C,
                           ctx->d_status, g.st);
@@ -373,7 +378,7 @@ cudaError_t stack_qr(dqmc_ctx* ctx, Group& g, double* Qt, double* Dv) {
     return launch_qr_blocked(g.X, g.nn(), Qt, g.sstride(), Dv, sD, g.Rtil, g.nn(), g.qrb, g.N, g.C,
                              g.oz, g.oz_batch, ctx->d_status, g.st, g.long_step);
   }
-  return launch_qrp_cluster(g.X, g.nn(), Qt, g.sstride(), Dv, sD, g.Rtil, g.nn(), g.qrs, g.N, g.C,
+  return launch_qrp_cluster(g.X, g.nn(), Qt, g.sstride(), Dv, sD, g.Rtil, g.nn(), g.N, g.C,
                             ctx->d_status, g.st);
 }
 
@@ -770,16 +775,17 @@ int setup_group(dqmc_ctx* ctx, Group& g) {
   DQ_RET(dev_alloc(ctx, &g.bins, C * (g.L + 1) * 2 * N * 8));
   DQ_RET(dev_alloc(ctx, &g.gacc, C * 3 * 8));
   DQ_RET(dev_alloc(ctx, &g.gout, C * (g.L + 1) * N * 8));
-  DQ_RET(dev_alloc(ctx, &g.qrs, C * 2 * N * 8));
   if (static_cast<int>(N) >= kOzakiMinN) {
     g.oz_batch = static_cast<int>(std::min<size_t>(C * S, 256));
     DQ_RET(dev_alloc(ctx, &g.oz, ozaki_scratch_bytes(static_cast<int>(N), g.oz_batch)));
-    DQ_RET(dev_alloc(ctx, &g.qrb.W0, C * NN * 8));
-    DQ_RET(dev_alloc(ctx, &g.qrb.W1, C * NN * 8));
-    DQ_RET(dev_alloc(ctx, &g.qrb.Wt, C * N * 32 * 8));
-    DQ_RET(dev_alloc(ctx, &g.qrb.perm, C * N * sizeof(int)));
-    g.qrb.sW = static_cast<long long>(NN);
-    g.qrb.sWt = static_cast<long long>(N) * 32;
+    if (qr_ctas(ctx, g) == 0) {  // stack_qr may take the blocked QR
+      DQ_RET(dev_alloc(ctx, &g.qrb.W0, C * NN * 8));
+      DQ_RET(dev_alloc(ctx, &g.qrb.W1, C * NN * 8));
+      DQ_RET(dev_alloc(ctx, &g.qrb.Wt, C * N * 32 * 8));
+      DQ_RET(dev_alloc(ctx, &g.qrb.perm, C * N * sizeof(int)));
+      g.qrb.sW = static_cast<long long>(NN);
+      g.qrb.sWt = static_cast<long long>(N) * 32;
+    }
   }
   std::vector<int> cpg = g.cp, cpd = g.cp;
   cpg.push_back(g.L + 1);

@@ -239,9 +239,7 @@ __device__ __forceinline__ int first_owned(int lo, int rank) {
 template <int CS>
 __global__ void __launch_bounds__(512) k_qrp_cluster(double* Xall, long long sX, double* Qall,
                                                     long long sQ, double* Dall, long long sD,
-                                                    double* Rall, long long sR, double* Vn, int n,
-                                                    int* status) {
-  (void)Vn;
+                                                    double* Rall, long long sR, int n, int* status) {
   cg::cluster_group cl = cg::this_cluster();
   const int rank = static_cast<int>(cl.block_rank());
   const int b = blockIdx.x / CS;
@@ -544,10 +542,9 @@ static cudaError_t launch_cluster(K kern, int cs, int batch, cudaStream_t st, Ar
 }
 
 cudaError_t launch_qrp_cluster(double* Xt, long long sX, double* Qt, long long sQ, double* D,
-                               long long sD, double* Rtil, long long sR, double* vnorm, int n,
-                               int batch, int* status, cudaStream_t st) {
-  return launch_cluster(k_qrp_cluster<2>, 2, batch, st, Xt, sX, Qt, sQ, D, sD, Rtil, sR, vnorm, n,
-                        status);
+                               long long sD, double* Rtil, long long sR, int n, int batch,
+                               int* status, cudaStream_t st) {
+  return launch_cluster(k_qrp_cluster<2>, 2, batch, st, Xt, sX, Qt, sQ, D, sD, Rtil, sR, n, status);
 }
 
 cudaError_t launch_gj_cluster(double* A, long long sA, double* Ainv, long long sI, int n, int batch,

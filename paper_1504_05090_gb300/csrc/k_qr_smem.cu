@@ -480,7 +480,7 @@ cudaError_t qs_launch(double* Xt, long long sX, double* Qt, long long sQ, double
 }  // namespace
 
 // CTAs per matrix of k_qr_smem, or 0 where another kernel takes the matrix.
-// The choice of kernel depends on n and the group's interval alone (stack_qr in
+// The choice of kernel depends on n and the group's interval alone (qr_ctas in
 // dqmc.cu), so that a chain's numbers do not depend on how many chains share its
 // context (the result does not depend on the CTAs either).  Measured (us for the
 // batch, GB300): this kernel against the blocked QR (the default mode's

@@ -142,10 +142,9 @@ cudaError_t launch_qrp(double* Xt, long long sX, double* Qt, long long sQ, doubl
 cudaError_t launch_gj_inverse(double* A, long long sA, int n, int batch, double* logabs,
                               double* sign, int* status, cudaStream_t st);
 // Cluster variants (k_cluster.cu): one 2-CTA cluster per matrix.
-// QR: vnorm is scratch of 2 n doubles per matrix.
 cudaError_t launch_qrp_cluster(double* Xt, long long sX, double* Qt, long long sQ, double* D,
-                               long long sD, double* Rtil, long long sR, double* vnorm, int n,
-                               int batch, int* status, cudaStream_t st);
+                               long long sD, double* Rtil, long long sR, int n, int batch,
+                               int* status, cudaStream_t st);
 // The same QR with the matrix in shared memory (k_qr_smem.cu), `cs` CTAs per
 // matrix: 1 (n <= 144), 4 or 8 (64 < n <= 144).  qr_smem_ctas gives the choice
 // for a context of `chains` chains (0: n is left to another kernel).
