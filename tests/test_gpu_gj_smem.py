@@ -48,3 +48,24 @@ def test_gtau_and_logw_match_oracle(Lx, Ly, prec):
         tol = 1e-10 if prec == "fp64" else 1e-9
         assert np.max(np.abs(sim.gtau()[0][1] - ref)) < tol * np.max(np.abs(ref))
         assert sim.grad()[2][1] == pytest.approx(ch.logw(), rel=1e-10)
+
+
+@pytest.mark.parametrize("Lx,Ly,counts", [(10, 6, (40, 80)), (8, 8, (40, 80)), (16, 8, (10, 40, 80)),
+                                          (16, 14, (10, 30, 60))])
+def test_every_chain_agrees_between_variants(Lx, Ly, counts):
+    """4 CTAs against one (N <= 144), 8 against 4, 4 against the matrix in global
+    memory (N = 224): every chain that the contexts share, U = 4, after a sweep."""
+    import paper_1504_05090_gb300 as pkg
+    ref = None
+    for C in counts:
+        g = pkg.Group(Lx=Lx, Ly=Ly, t=0.25, U=4.0, beta=5.0, dtau=0.25, n_chains=C, stab_interval=5,
+                      delay_k=8, precision="df32")
+        with pkg.DQMC([g], seed=9) as sim:
+            sim.sweep(1)
+            got = [sim.G(c, 0) for c in range(min(counts))]
+            f = sim.field()[0][:min(counts)]
+        if ref is None:
+            ref, f0 = got, f
+        assert np.array_equal(f, f0)
+        for x, y in zip(got, ref):
+            assert np.array_equal(x, y)

@@ -31,3 +31,27 @@ def test_green_of_every_panel_width_matches_oracle(Lx, Ly, C):
             ref = o.Chain(p, seed=21, chain=c).green(0, 1)
             G = sim.G(c, 0)
             assert np.max(np.abs(G - ref)) < 1e-10 * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("Lx,Ly,beta,dtau,ns", [(16, 10, 10.0, 0.1, 8), (14, 12, 8.0, 0.2, 6)])
+def test_blocked_qr_matches_pivoted_qr_above_144(Lx, Ly, beta, dtau, ns):
+    """Partial last panels (N = 160: 32 columns, 168: 8), swept fields: G, the
+    decisions of a sweep and G(tau) on the column-pivoted QR agree to 1e-10."""
+    import paper_1504_05090_gb300 as pkg
+    g = _grp(Lx, Ly, C=2, beta=beta, dtau=dtau, ns=ns, k=16)
+    with pkg.DQMC([g], seed=7) as a, pkg.DQMC([g], seed=7) as b:
+        b.set_qr_mode("pivoted")
+        a.sweep(2)
+        b.sweep(2)
+        b.set_field(a.field())
+        a.recompute_G()
+        for step in range(2):
+            for c in range(2):
+                Ga, Gb = a.G(c, 0), b.G(c, 0)
+                assert np.max(np.abs(Ga - Gb)) < 1e-10 * np.max(np.abs(Gb)), (step, c)
+            if step == 0:
+                a.sweep(1)
+                b.sweep(1)
+                assert np.array_equal(a.field()[0], b.field()[0])
+        x, y = a.gtau()[0], b.gtau()[0]
+        assert np.max(np.abs(x - y)) < 1e-10 * np.max(np.abs(y))
