@@ -172,6 +172,10 @@ __global__ void __launch_bounds__(kPT, 2) k_qrb_panel(const double* Wsall, long 
     src_of[rk] = static_cast<short>(i);
   }
   __syncthreads();
+  // columns too large for the sums to come: see kQsBig (keys: log2 of the squared
+  // norms, 3e38 for one that is not finite)
+  const float kmax = key[src_of[0]];
+  const bool big = kmax >= 1020.0f && kmax < 1.0e38f;
 
   // 2. the panel
   double x[kR];
@@ -185,6 +189,7 @@ __global__ void __launch_bounds__(kPT, 2) k_qrb_panel(const double* Wsall, long 
     for (int t = 0; t < kR; ++t) {
       const int r = lane + 32 * t;
       x[t] = (exists && r < m) ? Ws[static_cast<size_t>(c0 + src_of[cid]) * n + c0 + r] : 0.0;
+      if (big) x[t] *= kQsDown;
     }
     auto sumsq = [&](int j) {  // rows > j
       double a = (lane > j) ? x[0] * x[0] : 0.0;
@@ -433,11 +438,12 @@ __global__ void __launch_bounds__(kPT, 2) k_qrb_panel(const double* Wsall, long 
     const int q = step;
     double* d = Wd + static_cast<size_t>(c0 + q) * n;
     const double* s = Ws + static_cast<size_t>(c0 + src_of[cid]) * n;
-    if (lane <= q) d[c0 + lane] = (lane == q) ? betas[q] : x[0];
+    const double up = big ? kQsUp : 1.0;
+    if (lane <= q) d[c0 + lane] = ((lane == q) ? betas[q] : x[0]) * up;
     for (int r = lane; r < c0; r += 32) d[r] = s[r];  // entries above the panel
     if (lane == 0) {
       perm[c0 + q] = pold[src_of[cid]];
-      double dd = absd(betas[q]);
+      double dd = absd(betas[q]) * up;
       if (!(dd > 0.0) || !isfinite(dd)) {
         atomicExch(status, dd > 0.0 ? kDevNonFinite : kDevSingular);
         if (!(dd > 0.0)) dd = DBL_MIN;

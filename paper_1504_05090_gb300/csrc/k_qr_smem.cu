@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(kQT, 2) k_qr_smem(double* Xall, long long sX, 
   __shared__ unsigned char live[2][kMaxN / CS], rec[kMaxN / CS], colof[kMaxN / CS == kMaxN ? kMaxN : 1];
   __shared__ short stepof[kMaxN / CS];
   __shared__ Cand cand[2][CS];  // by step parity and CTA
-  __shared__ int wait_sum[2], stale[2];
+  __shared__ int wait_sum[2], stale[2], big_sh;
   __shared__ double kap_sh, vj_sh;
   __shared__ double vjs[CS == 1 ? kMaxN : 1];  // v_j[j]
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -130,6 +130,7 @@ __global__ void __launch_bounds__(kQT, 2) k_qr_smem(double* Xall, long long sX, 
   if (tid < 2) {
     wait_sum[tid] = 0;
     stale[tid] = -1;
+    big_sh = 0;
   }
   __syncthreads();
   for (int g = w; 8 * g < ncol; g += nw) {
@@ -145,6 +146,26 @@ __global__ void __launch_bounds__(kQT, 2) k_qr_smem(double* Xall, long long sX, 
   }
   __syncthreads();
   if constexpr (CS > 1) cl.sync();  // the peers run: their shared memory may be written
+  {  // columns too large for the sums to come: see kQsBig
+    int big = 0;
+    for (int i = tid; i < ncol; i += kQT) big |= key[i] >= kQsBig && key[i] < kQsNonFinite;
+    big = __syncthreads_or(big);
+    if (CS == 1) {
+      if (tid == 0) big_sh = big;
+    } else {
+      if (big && tid < CS) *cl.map_shared_rank(&big_sh, tid) = 1;
+      cl.sync();
+      big = big_sh;
+    }
+    if (big) {
+      for (int e = tid; e < ncol * ld; e += kQT) Xs[e] *= kQsDown;
+      for (int i = tid; i < ncol; i += kQT) {
+        n1[i] = n2[i] = n1[i] * (kQsDown * kQsDown);
+        key[i] = static_cast<unsigned>(__double2hiint(n1[i]));
+      }
+      __syncthreads();
+    }
+  }
 
   // Warp ws: own column lp (-1: none) brought to step j (upd: with the factor
   // of step j - 1 and its column xq), its sigma and, for CS > 1, both to every
@@ -439,7 +460,7 @@ __global__ void __launch_bounds__(kQT, 2) k_qr_smem(double* Xall, long long sX, 
       atomicExch(status, kDevSingular);
       d = DBL_MIN;
     }
-    if (rank == 0) D[i] = d;
+    if (rank == 0) D[i] = big_sh ? d * kQsUp : d;
     rd[i] = 1.0 / d;
   }
   __syncthreads();

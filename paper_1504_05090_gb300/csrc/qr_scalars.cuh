@@ -12,6 +12,15 @@ __device__ __forceinline__ double qs_scale2(double x, int e) {
   return __longlong_as_double(__double_as_longlong(x) + (static_cast<long long>(e) << 52));
 }
 
+// Squared norms from 2^1020 on (this high word): sums that the reflector needs,
+// up to twice the largest squared norm, could leave the range of FP64, and the
+// reciprocal its normal numbers, although the columns do neither.  The columns
+// are then scaled by kQsDown before the first step and R by kQsUp after the
+// last; no further down, as the smallest columns of such a product lie near the
+// lower end of the range.
+constexpr unsigned kQsBig = 2043u << 20, kQsNonFinite = 0x7FF00000u;
+constexpr double kQsDown = 0x1p-4, kQsUp = 0x1p4;
+
 // The leading 24 bits of a double in [1, 4) as a float, and a float as a
 // double, in integer arithmetic (a conversion would take the FP64 pipe).
 __device__ __forceinline__ float qs_to_f(double x) {
@@ -62,8 +71,9 @@ __device__ __forceinline__ void qs_reflector(double alpha, double sigma, double&
 // Warp sum of non-negative finite numbers in 64-bit fixed point: aligned to
 // the largest exponent (58 bits, rounded), three integer warp reductions
 // instead of five rounds of shuffles and FP64 additions (about 130 against 650
-// clocks).  Error below 2^-53 of the sum.  Non-finite input gives non-finite
-// output.
+// clocks).  Error below 2^-52 of the sum: up to 15.5 units of 2^-57 of the
+// largest term's power of two, and the rounding of the sum.  Non-finite input
+// gives non-finite output.
 __device__ __forceinline__ double qs_warp_sum_pos(double a) {
   const unsigned long long bits = static_cast<unsigned long long>(__double_as_longlong(a));
   const int E = static_cast<int>((bits >> 52) & 0x7FF);
@@ -89,7 +99,8 @@ __device__ __forceinline__ double qs_warp_sum_pos(double a) {
 }
 
 // The same for numbers of either sign: a bias of 2^58 per lane keeps the words
-// non-negative.  Error below 2^-54 of the largest term.
+// non-negative.  Error below 2^-53 of the largest term, and the rounding of the
+// sum.
 __device__ __forceinline__ double qs_warp_sum(double a) {
   const unsigned long long bits = static_cast<unsigned long long>(__double_as_longlong(a));
   const int E = static_cast<int>((bits >> 52) & 0x7FF);
