@@ -13,6 +13,7 @@ namespace dqmc {
 constexpr int kMaxSide = 16;
 constexpr int kMaxN = kMaxSide * kMaxSide;  // 256 sites
 constexpr int kMaxDelay = 32;
+constexpr int kSMs = 152;  // of a GB300, where a launcher without a context spreads work
 
 // ---------------------------------------------------------------------------
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11): 10 rounds of the

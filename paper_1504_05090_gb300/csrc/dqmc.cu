@@ -465,8 +465,9 @@ int form_mid(dqmc_ctx* ctx, Group& g, int j0, long long es, int batch, double* o
 }
 
 // Ainv = A^{-1} of `batch` middle matrices of the group (A may be
-// overwritten), `conc` of all groups' matrices in flight at once; pair:
-// eliminate in float pairs.
+// overwritten); conc: the matrices in flight at once, of all groups in a sweep
+// and of this group in a pass over its stabilisation points; pair: eliminate in
+// float pairs.
 cudaError_t invert(dqmc_ctx* ctx, Group& g, double* A, double* Ainv, int batch, long long conc,
                    double* logabs, bool pair) {
   const int cs = gj_smem_ctas(g.N, conc, ctx->nsm, pair);

@@ -721,7 +721,7 @@ cudaError_t launch_gemm(const GemmArgs& a, int batch, cudaStream_t st) {
   if (a.n < 64) {
     // rows per CTA: about two CTAs per SM for a small batch, whole matrices for
     // a large one (every CTA loads all of B)
-    const int parts = std::max(1, std::min((a.n + 1) / 2, 2 * 152 / batch));
+    const int parts = std::max(1, std::min((a.n + 1) / 2, 2 * kSMs / batch));
     const int R = (a.n + parts - 1) / parts;
     const size_t sm = (static_cast<size_t>(a.n) * (a.n | 1) + static_cast<size_t>(R) * a.n) * sizeof(double);
     cudaError_t e = cudaFuncSetAttribute(k_gemm_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -756,7 +756,7 @@ cudaError_t launch_set_identity(double* M, long long sM, double* D, long long sD
 
 template <typename T>
 cudaError_t launch_convert(const double* src, T* dst, long long n, cudaStream_t st) {
-  const int blocks = static_cast<int>(std::min<long long>((n + 255) / 256, 152 * 8));
+  const int blocks = static_cast<int>(std::min<long long>((n + 255) / 256, kSMs * 8));
   k_convert<T><<<std::max(blocks, 1), 256, 0, st>>>(src, dst, n);
   return cudaGetLastError();
 }

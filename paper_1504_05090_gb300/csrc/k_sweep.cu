@@ -795,23 +795,21 @@ struct alignas(2 * sizeof(T)) KronPair {
   T a, b;
 };
 
-// Tap t of a table (below).  Float pairs on even sides: taps 2i, 2i + 1 as
-// (hi, hi, lo, lo), so that one 16-byte load gives both packed operands.
+// Tap t of a table (below).  Float pairs: taps 2i, 2i + 1 as (hi, hi, lo, lo), so
+// that one 16-byte load gives both packed operands.
 template <typename T>
-__device__ __forceinline__ void kron_put_tap(T* tab, int t, double x, bool even) {
+__device__ __forceinline__ void kron_put_tap(T* tab, int t, double x) {
   if constexpr (std::is_same<T, df32>::value) {
-    if (even) {
-      const df32 d(x);
-      float* f = reinterpret_cast<float*>(tab) + 4 * (t >> 1) + (t & 1);
-      f[0] = d.hi;
-      f[2] = d.lo;
-      return;
-    }
+    const df32 d(x);
+    float* f = reinterpret_cast<float*>(tab) + 4 * (t >> 1) + (t & 1);
+    f[0] = d.hi;
+    f[2] = d.lo;
+  } else {
+    tab[t] = static_cast<T>(x);
   }
-  tab[t] = static_cast<T>(x);
 }
 
-// One side of the transform in float pairs, both sides even: two neighbouring
+// One side of the transform in float pairs: two neighbouring
 // outputs along the side are the two lanes of packed sums, and a thread takes
 // them for V vectors (vi, vi + nv / V), which share the tap load.  The same
 // operations in the same order per output as with scalar sums.
@@ -870,102 +868,59 @@ __device__ __forceinline__ void kron_transform(T* v, T* tmp, int nv, int ld, int
     }
     __syncthreads();
   }
-  if ((Lx & 1) == 0 && (Ly & 1) == 0) {
-    // Even sides: a thread takes two neighbouring outputs (x, x + 1) of one
-    // row (then (y, y + 1) of one column).  Both sums read the same input
-    // entry (one load), and their taps E[x - x'], E[x + 1 - x'] are adjacent:
-    // one 16-byte load from tx (tap index even) or from txs, the same taps
-    // shifted by one (odd).  Same additions in the same order per output.
-    if constexpr (std::is_same<T, df32>::value) {
-      if ((nv & 1) == 0 && nv * N >= 4 * static_cast<int>(blockDim.x)) {
-        kron_side_df32<2, false>(v, tmp, nv, ld, Lx, Ly, tx, txs, nullptr);
-        __syncthreads();
-        kron_side_df32<2, true>(tmp, v, nv, ld, Lx, Ly, ty, tys, post);
-      } else {
-        kron_side_df32<1, false>(v, tmp, nv, ld, Lx, Ly, tx, txs, nullptr);
-        __syncthreads();
-        kron_side_df32<1, true>(tmp, v, nv, ld, Lx, Ly, ty, tys, post);
-      }
+  // Both sides are even: a thread takes two neighbouring outputs (x, x + 1) of one
+  // row (then (y, y + 1) of one column).  Both sums read the same input
+  // entry (one load), and their taps E[x - x'], E[x + 1 - x'] are adjacent:
+  // one 16-byte load from tx (tap index even) or from txs, the same taps
+  // shifted by one (odd).  Same additions in the same order per output.
+  if constexpr (std::is_same<T, df32>::value) {
+    if ((nv & 1) == 0 && nv * N >= 4 * static_cast<int>(blockDim.x)) {
+      kron_side_df32<2, false>(v, tmp, nv, ld, Lx, Ly, tx, txs, nullptr);
       __syncthreads();
-      return;
-    }
-    const int hx = Lx >> 1, hy = Ly >> 1;
-    const int ptx = nv * Ly * hx;
-    for (int e = threadIdx.x; e < ptx; e += blockDim.x) {
-      const int vi = e / (Ly * hx), rr = e - vi * (Ly * hx), y = rr / hx, x = 2 * (rr - y * hx);
-      const T* row = v + vi * ld + Lx * y;
-      ProdSum<T> a0, a1;
-      for (int xp = 0; xp < Lx; ++xp) {
-        const int b = x + Lx - xp;  // tap index of output x; b + 1 that of x + 1
-        const KronPair<T> t2 = (b & 1) ? *reinterpret_cast<const KronPair<T>*>(txs + b - 1)
-                                       : *reinterpret_cast<const KronPair<T>*>(tx + b);
-        const T r = row[xp];
-        a0.add(t2.a, r);
-        a1.add(t2.b, r);
-      }
-      tmp[vi * ld + Lx * y + x] = a0.get();
-      tmp[vi * ld + Lx * y + x + 1] = a1.get();
-    }
-    __syncthreads();
-    const int pty = nv * hy * Lx;
-    for (int e = threadIdx.x; e < pty; e += blockDim.x) {
-      const int vi = e / (hy * Lx), rr = e - vi * (hy * Lx), yp2 = rr / Lx, x = rr - yp2 * Lx;
-      const int y = 2 * yp2;
-      const T* col = tmp + vi * ld + x;
-      ProdSum<T> a0, a1;
-      for (int yp = 0; yp < Ly; ++yp) {
-        const int b = y + Ly - yp;
-        const KronPair<T> t2 = (b & 1) ? *reinterpret_cast<const KronPair<T>*>(tys + b - 1)
-                                       : *reinterpret_cast<const KronPair<T>*>(ty + b);
-        const T c = col[Lx * yp];
-        a0.add(t2.a, c);
-        a1.add(t2.b, c);
-      }
-      const int i0 = x + Lx * y, i1 = i0 + Lx;
-      v[vi * ld + i0] = post ? a0.get() * post[i0] : a0.get();
-      v[vi * ld + i1] = post ? a1.get() * post[i1] : a1.get();
+      kron_side_df32<2, true>(tmp, v, nv, ld, Lx, Ly, ty, tys, post);
+    } else {
+      kron_side_df32<1, false>(v, tmp, nv, ld, Lx, Ly, tx, txs, nullptr);
+      __syncthreads();
+      kron_side_df32<1, true>(tmp, v, nv, ld, Lx, Ly, ty, tys, post);
     }
     __syncthreads();
     return;
   }
-  // A thread takes the same element of two vectors (2 vp, 2 vp + 1): the two
-  // sums are independent and share every tap load.  The taps are stored twice
-  // over (tx[k] = Ex[k mod Lx] for k < 2 Lx), so that tap x - x' mod Lx is
-  // tx[x + Lx - x'] without a wrap test.
-  const int npair = (nv + 1) >> 1, ptot = npair * N;
-  for (int e = threadIdx.x; e < ptot; e += blockDim.x) {
-    const int vp = e / N, i = e - vp * N;
-    const int x = i % Lx, y = i / Lx;
-    const bool two = 2 * vp + 1 < nv;
-    const T* row0 = v + (2 * vp) * ld + Lx * y;
-    const T* row1 = two ? row0 + ld : row0;
-    const T* tp = tx + x + Lx;
+  const int hx = Lx >> 1, hy = Ly >> 1;
+  const int ptx = nv * Ly * hx;
+  for (int e = threadIdx.x; e < ptx; e += blockDim.x) {
+    const int vi = e / (Ly * hx), rr = e - vi * (Ly * hx), y = rr / hx, x = 2 * (rr - y * hx);
+    const T* row = v + vi * ld + Lx * y;
     ProdSum<T> a0, a1;
     for (int xp = 0; xp < Lx; ++xp) {
-      const T t = tp[-xp];
-      a0.add(t, row0[xp]);
-      a1.add(t, row1[xp]);
+      const int b = x + Lx - xp;  // tap index of output x; b + 1 that of x + 1
+      const KronPair<T> t2 = (b & 1) ? *reinterpret_cast<const KronPair<T>*>(txs + b - 1)
+                                     : *reinterpret_cast<const KronPair<T>*>(tx + b);
+      const T r = row[xp];
+      a0.add(t2.a, r);
+      a1.add(t2.b, r);
     }
-    tmp[(2 * vp) * ld + i] = a0.get();
-    if (two) tmp[(2 * vp + 1) * ld + i] = a1.get();
+    tmp[vi * ld + Lx * y + x] = a0.get();
+    tmp[vi * ld + Lx * y + x + 1] = a1.get();
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < ptot; e += blockDim.x) {
-    const int vp = e / N, i = e - vp * N;
-    const int x = i % Lx, y = i / Lx;
-    const bool two = 2 * vp + 1 < nv;
-    const T* col0 = tmp + (2 * vp) * ld + x;
-    const T* col1 = two ? col0 + ld : col0;
-    const T* tp = ty + y + Ly;
+  const int pty = nv * hy * Lx;
+  for (int e = threadIdx.x; e < pty; e += blockDim.x) {
+    const int vi = e / (hy * Lx), rr = e - vi * (hy * Lx), yp2 = rr / Lx, x = rr - yp2 * Lx;
+    const int y = 2 * yp2;
+    const T* col = tmp + vi * ld + x;
     ProdSum<T> a0, a1;
     for (int yp = 0; yp < Ly; ++yp) {
-      const T t = tp[-yp];
-      a0.add(t, col0[Lx * yp]);
-      a1.add(t, col1[Lx * yp]);
+      const int b = y + Ly - yp;
+      const KronPair<T> t2 = (b & 1) ? *reinterpret_cast<const KronPair<T>*>(tys + b - 1)
+                                     : *reinterpret_cast<const KronPair<T>*>(ty + b);
+      const T c = col[Lx * yp];
+      a0.add(t2.a, c);
+      a1.add(t2.b, c);
     }
-    const T sc = post ? post[i] : T(1);
-    v[(2 * vp) * ld + i] = post ? a0.get() * sc : a0.get();
-    if (two) v[(2 * vp + 1) * ld + i] = post ? a1.get() * sc : a1.get();
+    const int i0 = x + Lx * y, i1 = i0 + Lx;
+    v[vi * ld + i0] = post ? a0.get() * post[i0] : a0.get();
+    v[vi * ld + i1] = post ? a1.get() * post[i1] : a1.get();
   }
   __syncthreads();
 }
@@ -1015,12 +970,12 @@ template <typename T>
 __device__ __forceinline__ void kron_load_taps(const KronArgs& a, KronStage<T> s) {
   if (threadIdx.x < 2 * kMaxSide) {  // each circulant row twice over (kron_transform)
     const int t = threadIdx.x, tx = t % a.Lx, ty = t % a.Ly;
-    const bool inv = (a.kind == kBIT), ev = ((a.Lx | a.Ly) & 1) == 0;
+    const bool inv = (a.kind == kBIT);
     const int tx1 = (t + 1) % a.Lx, ty1 = (t + 1) % a.Ly;
-    kron_put_tap(s.tx, t, inv ? a.taps.exi[tx] : a.taps.ex[tx], ev);
-    kron_put_tap(s.ty, t, inv ? a.taps.eyi[ty] : a.taps.ey[ty], ev);
-    kron_put_tap(s.txs, t, inv ? a.taps.exi[tx1] : a.taps.ex[tx1], ev);
-    kron_put_tap(s.tys, t, inv ? a.taps.eyi[ty1] : a.taps.ey[ty1], ev);
+    kron_put_tap(s.tx, t, inv ? a.taps.exi[tx] : a.taps.ex[tx]);
+    kron_put_tap(s.ty, t, inv ? a.taps.eyi[ty] : a.taps.ey[ty]);
+    kron_put_tap(s.txs, t, inv ? a.taps.exi[tx1] : a.taps.ex[tx1]);
+    kron_put_tap(s.tys, t, inv ? a.taps.eyi[ty1] : a.taps.ey[ty1]);
   }
 }
 
@@ -1138,15 +1093,14 @@ __global__ void __launch_bounds__(kWT, 2) k_wrap_smem(T* X, KronArgs a) {
   }
   if (threadIdx.x < 2 * kMaxSide) {  // each circulant row twice over (kron_transform)
     const int t = threadIdx.x, tx = t % a.Lx, ty = t % a.Ly, tx1 = (t + 1) % a.Lx, ty1 = (t + 1) % a.Ly;
-    const bool ev = ((a.Lx | a.Ly) & 1) == 0;
-    kron_put_tap(s.tx, t, a.taps.ex[tx], ev);
-    kron_put_tap(s.ty, t, a.taps.ey[ty], ev);
-    kron_put_tap(s.txs, t, a.taps.ex[tx1], ev);
-    kron_put_tap(s.tys, t, a.taps.ey[ty1], ev);
-    kron_put_tap(taps2, t, a.taps.exi[tx], ev);
-    kron_put_tap(taps2 + 2 * kMaxSide, t, a.taps.eyi[ty], ev);
-    kron_put_tap(taps2 + 4 * kMaxSide, t, a.taps.exi[tx1], ev);
-    kron_put_tap(taps2 + 6 * kMaxSide, t, a.taps.eyi[ty1], ev);
+    kron_put_tap(s.tx, t, a.taps.ex[tx]);
+    kron_put_tap(s.ty, t, a.taps.ey[ty]);
+    kron_put_tap(s.txs, t, a.taps.ex[tx1]);
+    kron_put_tap(s.tys, t, a.taps.ey[ty1]);
+    kron_put_tap(taps2, t, a.taps.exi[tx]);
+    kron_put_tap(taps2 + 2 * kMaxSide, t, a.taps.eyi[ty]);
+    kron_put_tap(taps2 + 4 * kMaxSide, t, a.taps.exi[tx1]);
+    kron_put_tap(taps2 + 6 * kMaxSide, t, a.taps.eyi[ty1]);
   }
   const T up = static_cast<T>(a.ec), dn = static_cast<T>(a.emc);
   const int8_t* f = a.field + (static_cast<size_t>(b) * a.L + a.l0_first) * N;
@@ -1429,7 +1383,7 @@ __global__ void __launch_bounds__(256) k_corr_length(const double* spin, const d
 cudaError_t launch_init_field(int8_t* field, int C, int L, int N, int chain0, uint64_t seed,
                               cudaStream_t st) {
   const long long total = static_cast<long long>(C) * L * N;
-  const int blocks = static_cast<int>(std::min<long long>((total + 255) / 256, 152 * 16));
+  const int blocks = static_cast<int>(std::min<long long>((total + 255) / 256, kSMs * 16));
   k_init_field<<<blocks, 256, 0, st>>>(field, C, L, N, chain0, static_cast<uint32_t>(seed),
                                        static_cast<uint32_t>(seed >> 32));
   return cudaGetLastError();
