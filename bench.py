@@ -233,10 +233,11 @@ DF32_PEAK = 2 * 152 * 128 * 2.07e9 / 14 / 1e12
 # counters were taken: if a file has changed since, the entry is stale and the
 # roofline line reports null.  (profiles/launches_profile_case_16x16.md)
 TRAFFIC = {
-    # panel x 8, fused rank-32 products x 30, finalize: one blocked QR launch
-    ("qr_pivot", None): (687.3e6, ("k_qr_blocked.cu", "k_ozaki.cu"), "443fe89b26ebd644"),
-    ("metropolis", "df32"): (33.67e6, ("k_sweep.cu",), "a31adbbee642dc65"),
-    ("stack_kron", None): (34.09e6, ("k_kron_tc.cu",), "33ed7cfa2a480480"),
+    # panel x 8, rank-32 products x 30 (six of them in one CTA per matrix), finalize:
+    # one blocked QR launch
+    ("qr_pivot", None): (687.3e6, ("k_qr_blocked.cu", "qr_scalars.cuh", "k_ozaki.cu"), "2425d8c3e0d31642"),
+    ("metropolis", "df32"): (33.66e6, ("k_sweep.cu",), "ff1c9aa5e8d7ae31"),
+    ("stack_kron", None): (34.05e6, ("k_kron_tc.cu",), "e89bcb6e4ae4de21"),
 }
 
 

@@ -176,15 +176,16 @@ constexpr double kTuneMargin = 0.05;  // probe drift must stay below 5% of the t
 // the columns of a stack step over n slices spread by up to e^{2 n (lambda +
 // 4 |t| dtau)}, and the rounding of the step comes out of it amplified.  Two
 // FP64-accurate ways to form the stacks then give G(tau) that differ, in the
-// worst entry relative to its RMS (8 x 8, 128 chains; 10 x 10, 96), by
-//   exponent 12.7: 6e-12, 8e-12    13.7: 1e-11, 7e-11    17.2: 9e-10, 2e-9
-//            20.5: 6e-10, 2e-9     21.7: 1e-8, 1e-8 (7e-8 over more chains)
+// worst entry relative to its RMS (8 x 8, 512 chains; 12 x 12, 96), by
+//   exponent 12.7: 1e-11, 6e-12      16.0 (U = 4): 2e-9, 7e-9
+//            18.7 (U = 4): 7e-9, 4e-8    21.7 (U = 2): 2e-8 to 7e-8, 3e-8
 // in FP64 and float-pair groups alike.  Beyond kLongStep such a difference is
-// no longer small, and it is as large against the exact value whichever way is
-// taken.  The groups there keep the kernels that their stacks have always been
-// formed by, operation for operation, so that G(tau) of a field is reproduced:
-// k_qrp_cluster (N < 64), panels of two CTAs and Kronecker products of eight
-// digits.  A common interval (n_s dtau = 1.25, U <= 3) has 12 to 15.
+// no longer small, and each way is as far from the exact value.  The groups
+// there keep the kernels that their stacks have always been formed by, operation
+// for operation, so that G(tau) of a field is reproduced: k_qrp_cluster (N < 64),
+// panels of two CTAs and Kronecker products of eight digits.  That costs time (8 x
+// 8, three groups of 256 chains, one of them at 21.7: 116 -> 136 ms a sweep).  A
+// common interval (n_s dtau = 1.25, U <= 3) has 12 to 16.
 constexpr double kLongStep = 16.0;
 bool stretches_far(const dqmc_group& p, int L, double lam) {
   return 2.0 * std::min(p.stab_interval, L) * (lam + 4.0 * std::fabs(p.t) * p.dtau) > kLongStep;
