@@ -1,11 +1,13 @@
 // Panels of the blocked QR (k_qr_blocked.cu) with the rows of a panel split
 // between the two CTAs of a cluster and its columns in shared memory.
 //
-// The panels of k_qrb_panel are faster (64 matrices of order 64 580 us with
-// these, of order 256 3.49 ms against 2.71); these stay for the groups whose
-// stack steps stretch a vector so far that single entries of G(tau) carry the
-// rounding of a step amplified to 1e-8 and more (long_step in dqmc.cu): the
-// order of every sum here is part of their numbers.
+// Bound by the chain of Householder steps, two exchanges between the CTAs each.
+// Others are faster (a whole QR of 32 matrices of order 64: 580 us with these,
+// 258 in shared memory; 64 of order 256: 3.49 ms against 2.71 with k_qrb_panel);
+// these stay for the groups whose stack steps stretch a vector so far that
+// single entries of G(tau) carry the rounding of a step amplified to 1e-8 and
+// more (long_step in dqmc.cu): the order of every sum here is part of their
+// numbers.
 #include <cooperative_groups.h>
 
 #include <cfloat>
